@@ -62,9 +62,12 @@ enum {
   DMRG2D_TF32 = 1,   /* v float, y float; tcgen05 kind::tf32, FP32 accumulate in TMEM */
   DMRG2D_BF16 = 2,   /* v bf16 (uint16 bits), y float; tcgen05 kind::f16, FP32 acc  */
   DMRG2D_FP32 = 3,   /* v float, y float; FP32 FMA on CUDA cores                      */
-  DMRG2D_FP64X = 4,  /* v, y double; float-pair arithmetic (~48-bit significands) on
-                        the FP32 CUDA cores: FP64 emulated for the mixed solver's
-                        residuals (sector layouts: the scalar moves in FP64)         */
+  DMRG2D_FP64X = 4,  /* v, y double; FP64 emulated for the mixed solver's residuals: the
+                        entries of v and of the operator blocks as integers of 52 bits
+                        below the largest entry of their row (of H_l, H_r) or line (of
+                        V), multiplied exactly in FP16 digits on the tensor cores;
+                        products below 2^-52 of the largest one are left out.  Scalar
+                        moves in FP64.  A non-finite entry gives NaN                 */
   DMRG2D_BF16X3 = 5  /* split BF16: v = [v_hi | v_lo], 2 n_vec bf16 values with
                         v_hi = bf16(x), v_lo = bf16(x - v_hi) (dmrg2d_convert_input);
                         y float; three BF16 tensor-core products into FP32,
@@ -184,7 +187,7 @@ typedef struct dmrg2d_solver_opts {
                           start (2 = full reorthogonalisation as in the plain solve,
                           1 = one pass, 0 = the three-term recurrence only)          */
   int refine_precision;/* mixed: H·v of the outer loop's residuals, DMRG2D_FP64 or
-                          DMRG2D_FP64X (float pairs)                                 */
+                          DMRG2D_FP64X                                               */
   int thick_keep;      /* plain Lanczos, at a full basis: 0 = explicit restart from the
                           lowest Ritz vector; p in 1..32 = thick restart (Wu and Simon)
                           keeping the p lowest Ritz vectors and the next Lanczos vector,
@@ -426,7 +429,7 @@ void dmrg2d_free_ops(dmrg2d_ops* ops);
  * returns last.
  * Ground states: `precision` FP64 runs the plain Lanczos (thick restart keeping
  * krylov_dim / 4 Ritz vectors, at most 16); TF32/BF16/BF16X3 the mixed solver with FP64
- * refinement (its outer-loop H·v in float pairs, DMRG2D_FP64X) where the tensor-core path
+ * refinement (its outer-loop H·v in DMRG2D_FP64X) where the tensor-core path
  * supports the superblock's shapes (plain FP64 otherwise).  solver =
  * DMRG2D_SWEEP_DAVIDSON takes dmrg2d_davidson_ground instead (basis of krylov_dim
  * vectors, clamped to 4..48; max_iter Davidson steps; with TF32/BF16/BF16X3

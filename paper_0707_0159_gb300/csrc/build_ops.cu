@@ -18,6 +18,7 @@
 #include <thread>
 
 #include "common.h"
+#include "longplan.h"
 
 namespace dmrg2d {
 
@@ -397,6 +398,34 @@ static int assemble(const dmrg2d_model* M, const dmrg2d_block* L, const dmrg2d_b
   return DMRG2D_OK;
 }
 
+// Work lists of the two-pass H·v for a dense superblock: one matrix, the block rows of H_l
+// and the block columns of H_r as segments.
+static int long_prepare(dmrg2d_ops* ops, cudaStream_t s) {
+  const int d = ops->d, m1 = ops->m1, m4 = ops->m4, ld = (int)ops->ld;
+  LongPlan* L = new LongPlan();
+  ops->lp = L;
+  const DeviceOps& D = ops->dev;
+  L->op64[0] = D.HR64;
+  L->op64[1] = D.HL64;
+  L->op32[0] = D.HR32;
+  L->op32[1] = D.HL32;
+  for (int i = 0; i < d; ++i) {
+    L->segs[0].push_back({0, ld, ld, i * m4, m4, m4, ops->hRptr[i], ops->hRptr[i + 1], 0, 0, 0, 0});
+    L->segs[1].push_back({0, ld, d * m4, i * m1, m1, m1, ops->hLptr[i], ops->hLptr[i + 1], 0, 0, 0,
+                          0});
+  }
+  for (int e = 0; e < D.nR; ++e) L->ks[0].push_back({(long long)e * m4 * m4, ops->hRcol[e] * m4, m4});
+  for (int e = 0; e < D.nL; ++e) L->ks[1].push_back({(long long)e * m1 * m1, ops->hLcol[e] * m1, m1});
+  auto at = [&](int t) { return (long long)(t % d) * m1 + (long long)ld * (t / d) * m4; };
+  for (int t = 0; t < d * d; ++t)
+    if (ops->hCptr[t + 1] > ops->hCptr[t])
+      lp_add_moves(L, at(t), ld, m1, m1, m4, ops->hCptr[t], ops->hCptr[t + 1]);
+  for (int e = 0; e < D.nC; ++e)
+    L->mrec.push_back({at(ops->hCsrc[e]), ld, (float)ops->hCval[e], ops->hCval[e]});
+  L->quads = m1 % 4 == 0;
+  return lp_finalise(ops, L, s);
+}
+
 static void release_device(dmrg2d_ops* ops) {
   DeviceOps& D = ops->dev;
   void* ptrs[] = {D.Lptr, D.Lcol, D.HL64, D.HL32, D.HL16, D.Rptr, D.Rcol,  D.HR64,
@@ -445,6 +474,7 @@ extern "C" int dmrg2d_build_ops(const dmrg2d_model* model, const dmrg2d_block* l
   if (target) {  // sector-restricted: pack the sub-blocks, skip the dense uploads
     st = sec_build(ops, left, right, target, HL, HR, s);
     if (st != DMRG2D_OK) {
+      lp_release(ops->lp);
       sec_release(ops);
       delete ops;
       return st;
@@ -481,8 +511,10 @@ extern "C" int dmrg2d_build_ops(const dmrg2d_model* model, const dmrg2d_block* l
     cudaError_t e = cudaStreamSynchronize(s);
     if (e != cudaSuccess) st = set_error(DMRG2D_ECUDA, "upload: %s", cudaGetErrorString(e));
   }
+  if (st == DMRG2D_OK) st = long_prepare(ops, s);
   if (st == DMRG2D_OK) st = tc_prepare(ops, s, HL, HR);
   if (st != DMRG2D_OK) {
+    lp_release(ops->lp);
     tc_release(ops);
     release_device(ops);
     delete ops;
@@ -558,6 +590,7 @@ extern "C" int dmrg2d_profile_stop(dmrg2d_ops* ops, double* total_ms, int* launc
 extern "C" void dmrg2d_free_ops(dmrg2d_ops* ops) {
   if (!ops) return;
   prof_clear(ops);
+  lp_release(ops->lp);
   sec_release(ops);
   tc_release(ops);
   release_device(ops);

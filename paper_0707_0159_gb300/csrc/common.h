@@ -77,6 +77,8 @@ struct DeviceOps {
   float* Cval32 = nullptr;
 };
 
+struct LongPlan;
+
 }  // namespace dmrg2d
 
 struct dmrg2d_ops {
@@ -94,6 +96,8 @@ struct dmrg2d_ops {
   std::vector<int> hqc;  // column quantum numbers, (N_up, N_dn) per column state
   // diagonal of H: H_l diagonal per (i1 + m1 i2), H_r per (i4 + m4 i3), H_c per (i2 + d i3)
   std::vector<double> hdL, hdR, hdC;
+  // work lists of the two-pass H·v (longplan.h)
+  dmrg2d::LongPlan* lp = nullptr;
   // sector-restricted operation (NULL for the dense superblock), opaque here
   void* sec = nullptr;
   // tensor-core path state (tensor maps of the operator blocks), opaque here

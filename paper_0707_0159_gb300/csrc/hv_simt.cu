@@ -8,7 +8,7 @@
 //   3. scalar moves (H_c and off-diagonal column terms): acc += c * V_tile(i2', i3')
 // and writes Y once.  V is column-major with leading dimension m1*d.
 #include "common.h"
-#include "ff.cuh"
+#include "longplan.h"
 
 namespace dmrg2d {
 
@@ -156,124 +156,6 @@ hv_simt_kernel(const T* __restrict__ v, T* __restrict__ y, const T* __restrict__
     }
 }
 
-// ---- FP64 emulated with float pairs (FP64X, ff.cuh) ------------------------------------
-// Same tiling as hv_simt_kernel; float-pair arithmetic runs on the FP32 pipes (64x the
-// FP64 rate on this part).
-__global__ void __launch_bounds__(TX * TY)
-hv_simt_ff_kernel(const double* __restrict__ v, double* __restrict__ y,
-                  const double* __restrict__ HL, const double* __restrict__ HR,
-                  const double* __restrict__ Cval, SimtParams p) {
-  __shared__ ff As[BK][BM];
-  __shared__ ff Bs[BK][BN];
-  const int nbm = (p.m1 + BM - 1) / BM;
-  const int nbn = (p.m4 + BN - 1) / BN;
-  const int bm = blockIdx.x % nbm, i2 = blockIdx.x / nbm;
-  const int bn = blockIdx.y % nbn, i3 = blockIdx.y / nbn;
-  const int i0 = bm * BM, j0 = bn * BN;
-  const int tid = threadIdx.x;
-  const int tx = tid % TX, ty = tid / TX;
-  const int m1 = p.m1, m4 = p.m4;
-  const int64_t ld = p.ld;
-  const ff zero = {0.f, 0.f};
-
-  ff acc[4][4];
-#pragma unroll
-  for (int a = 0; a < 4; ++a)
-#pragma unroll
-    for (int b = 0; b < 4; ++b) acc[a][b] = zero;
-
-  auto mma_tile = [&]() {
-#pragma unroll
-    for (int k = 0; k < BK; ++k) {
-      ff av[4], bv[4];
-#pragma unroll
-      for (int a = 0; a < 4; ++a) av[a] = As[k][tx + TX * a];
-#pragma unroll
-      for (int b = 0; b < 4; ++b) bv[b] = Bs[k][ty + TY * b];
-#pragma unroll
-      for (int a = 0; a < 4; ++a)
-#pragma unroll
-        for (int b = 0; b < 4; ++b) ff_fma(acc[a][b], av[a], bv[b]);
-    }
-  };
-
-  // ---- phase 1: H_l V ----
-  for (int e = p.Lptr[i2]; e < p.Lptr[i2 + 1]; ++e) {
-    const double* A = HL + (size_t)e * m1 * m1;
-    const double* B = v + (int64_t)p.Lcol[e] * m1 + ld * ((int64_t)i3 * m4);
-    for (int k0 = 0; k0 < m1; k0 += BK) {
-#pragma unroll
-      for (int r = 0; r < 4; ++r) {
-        const int k = tid % BK, i = tid / BK + 16 * r;
-        const int gi = i0 + i, gk = k0 + k;
-        As[k][i] = (gi < m1 && gk < m1) ? ff_of(A[(size_t)gi * m1 + gk]) : zero;
-        const int gj = j0 + i;
-        Bs[k][i] = (gk < m1 && gj < m4) ? ff_of(B[gk + ld * gj]) : zero;
-      }
-      __syncthreads();
-      mma_tile();
-      __syncthreads();
-    }
-  }
-  // ---- phase 2: V H_r^T ----
-  for (int e = p.Rptr[i3]; e < p.Rptr[i3 + 1]; ++e) {
-    const double* A = v + (int64_t)i2 * m1 + ld * ((int64_t)p.Rcol[e] * m4);
-    const double* B = HR + (size_t)e * m4 * m4;
-    for (int k0 = 0; k0 < m4; k0 += BK) {
-#pragma unroll
-      for (int r = 0; r < 4; ++r) {
-        const int i = tid % BM, k = tid / BM + 4 * r;
-        const int gi = i0 + i, gk = k0 + k;
-        As[k][i] = (gi < m1 && gk < m4) ? ff_of(A[gi + ld * gk]) : zero;
-        const int kb = tid % BK, j = tid / BK + 16 * r;
-        const int gj = j0 + j, gkb = k0 + kb;
-        Bs[kb][j] = (gj < m4 && gkb < m4) ? ff_of(B[(size_t)gj * m4 + gkb]) : zero;
-      }
-      __syncthreads();
-      mma_tile();
-      __syncthreads();
-    }
-  }
-  // ---- phase 3: scalar tile moves, then the single store of Y ----
-  const int t = i2 + p.d * i3;
-  for (int e = p.Cptr[t]; e < p.Cptr[t + 1]; ++e) {
-    const int src = p.Csrc[e];
-    const int s2 = src % p.d, s3 = src / p.d;
-    const ff c = ff_of(Cval[e]);
-    const double* S = v + (int64_t)s2 * m1 + ld * ((int64_t)s3 * m4);
-#pragma unroll
-    for (int a = 0; a < 4; ++a)
-#pragma unroll
-      for (int b = 0; b < 4; ++b) {
-        const int gi = i0 + tx + TX * a, gj = j0 + ty + TY * b;
-        if (gi < m1 && gj < m4) ff_fma(acc[a][b], c, ff_of(S[gi + ld * gj]));
-      }
-  }
-  double* Yt = y + (int64_t)i2 * m1 + ld * ((int64_t)i3 * m4);
-#pragma unroll
-  for (int a = 0; a < 4; ++a)
-#pragma unroll
-    for (int b = 0; b < 4; ++b) {
-      const int gi = i0 + tx + TX * a, gj = j0 + ty + TY * b;
-      if (gi < m1 && gj < m4) Yt[gi + ld * gj] = ff_to_double(acc[a][b]);
-    }
-}
-
-SimtParams simt_params(const dmrg2d_ops* ops) {
-  SimtParams p;
-  p.m1 = ops->m1;
-  p.m4 = ops->m4;
-  p.d = ops->d;
-  p.ld = ops->ld;
-  p.Lptr = ops->dev.Lptr;
-  p.Lcol = ops->dev.Lcol;
-  p.Rptr = ops->dev.Rptr;
-  p.Rcol = ops->dev.Rcol;
-  p.Cptr = ops->dev.Cptr;
-  p.Csrc = ops->dev.Csrc;
-  return p;
-}
-
 template <typename T>
 int launch(const dmrg2d_ops* ops, const T* v, T* y, const T* HL, const T* HR, const T* C,
            cudaStream_t s) {
@@ -318,27 +200,19 @@ int launch(const dmrg2d_ops* ops, const T* v, T* y, const T* HL, const T* HR, co
   return DMRG2D_OK;
 }
 
-int launch_ff(const dmrg2d_ops* ops, const double* v, double* y, cudaStream_t s) {
-  const SimtParams p = simt_params(ops);
-  const int64_t gx = (int64_t)((ops->m1 + BM - 1) / BM) * ops->d;
-  const int64_t gy = (int64_t)((ops->m4 + BN - 1) / BN) * ops->d;
-  if (gx > 0x7fffffff || gy > 65535)
-    return set_error(DMRG2D_EUNSUPPORTED, "SIMT grid %lld x %lld too large", (long long)gx,
-                     (long long)gy);
+int launch_fx(const dmrg2d_ops* ops, const double* v, double* y, cudaStream_t s) {
   auto ev = prof_slot(ops);
   if (ev.first) D2_CUDA(cudaEventRecord(ev.first, s));
-  hv_simt_ff_kernel<<<dim3((unsigned)gx, (unsigned)gy), TX * TY, 0, s>>>(
-      v, y, ops->dev.HL64, ops->dev.HR64, ops->dev.Cval64, p);
-  D2_CUDA(cudaGetLastError());
+  D2_TRY(fx_launch(ops->lp, v, y, s));
   if (ev.second) D2_CUDA(cudaEventRecord(ev.second, s));
-  return DMRG2D_OK;
+  return lp_moves_f64(ops->lp, v, y, s);
 }
 
 }  // namespace
 
 int launch_hv_simt_ff64(const dmrg2d_ops* ops, const double* v, double* y, cudaStream_t s) {
   if (ops->sec) return sec_apply(ops, v, y, DMRG2D_FP64X, s);
-  return launch_ff(ops, v, y, s);
+  return launch_fx(ops, v, y, s);
 }
 
 int launch_hv_simt_f64(const dmrg2d_ops* ops, const double* v, double* y, cudaStream_t s) {

@@ -23,6 +23,7 @@
 
 #include "common.h"
 #include "grouped.h"
+#include "longplan.h"
 #include "tc_ptx.cuh"
 
 namespace dmrg2d {
@@ -1131,6 +1132,9 @@ int tc_read_error(const dmrg2d_ops* ops, int* code) {
   int c3 = 0;
   D2_TRY(sec_read_error(ops, &c3));
   if (!*code) *code = c3;
+  int c4 = 0;
+  D2_TRY(lp_read_error(ops->lp, &c4));
+  if (!*code) *code = c4;
   return DMRG2D_OK;
 }
 

@@ -23,7 +23,6 @@
 #include <map>
 
 #include "common.h"
-#include "ff.cuh"
 #include "grouped.h"
 #include "longplan.h"
 
@@ -34,8 +33,6 @@ namespace {
 using Lab = std::array<int, 2>;
 Lab add(Lab a, Lab b) { return {a[0] + b[0], a[1] + b[1]}; }
 Lab sub(Lab a, Lab b) { return {a[0] - b[0], a[1] - b[1]}; }
-
-constexpr int SBM = 64, SBN = 64, SBK = 16;  // CUDA-core tile
 
 struct RowSegD {  // device row segment
   int q, off, dim, dim_pad, k1b, k1e;
@@ -55,10 +52,6 @@ struct K2D {  // phase 2: A = columns of V_q, B = R sub-block
   int a_col;        // first column of segment (i3', b') in V_q
   int kdim;
 };
-struct TileD {
-  int rs, cs;       // row / column segment
-  int r_in, c_in;   // first row / column inside the segments
-};
 struct MoveDst {
   int rs, cs, mb, me;
 };
@@ -67,30 +60,6 @@ struct MoveSrc {
   double c64;
   float c32;
 };
-struct MoveRec {    // a move as the kernel reads it: first element and ld of its source
-  long long src;
-  int ld;
-  float c32;
-  double c64;
-};
-struct MoveItem {   // columns c_in .. c_in + ncol of a destination sub-block
-  long long dst;    // its first element there
-  int ld, dim, nquad;  // leading dimension, rows, rows in fours with padding
-  int c_in, ncol, mb, me;
-};
-
-struct SecParams {
-  const long long* qbase;
-  const int* qld;
-  const RowSegD* rseg;
-  const ColSegD* cseg;
-  const K1D* k1;
-  const K2D* k2;
-  const TileD* tiles;
-  const MoveRec* mrec;
-  const MoveItem* mitems;
-};
-
 struct SecState {
   int nQ = 0;
   std::vector<long long> qbase;
@@ -99,24 +68,11 @@ struct SecState {
   std::vector<ColSegD> cseg;
   std::vector<K1D> k1;
   std::vector<K2D> k2;
-  std::vector<TileD> tiles;
   std::vector<MoveDst> mdst;
   std::vector<MoveSrc> msrc;
-  std::vector<MoveRec> mrec;
-  std::vector<MoveItem> mitems;
-  LongPlan lplan;  // two-pass CUDA-core form of the same work
   std::vector<int> rs_i2, rs_a, cs_i3, cs_b;  // host: segment identities
   std::vector<int> a_first, b_first;          // first state of each block sector
   // device copies
-  long long* d_qbase = nullptr;
-  int* d_qld = nullptr;
-  RowSegD* d_rseg = nullptr;
-  ColSegD* d_cseg = nullptr;
-  K1D* d_k1 = nullptr;
-  K2D* d_k2 = nullptr;
-  TileD* d_tiles = nullptr;
-  MoveRec* d_mrec = nullptr;
-  MoveItem* d_mitems = nullptr;
   double* d_L64 = nullptr;
   float* d_L32 = nullptr;
   double* d_R64 = nullptr;
@@ -129,178 +85,9 @@ struct SecState {
   std::vector<void*> allocs;
   GroupPlan plan;  // tensor-core form of the same work (pools deduplicated up to sign)
   bool gp_ok = false;
-
-  SecParams params() const {
-    return {d_qbase, d_qld, d_rseg, d_cseg, d_k1, d_k2, d_tiles, d_mrec, d_mitems};
-  }
 };
 
 // ---- kernels ------------------------------------------------------------------------------
-// T: storage type of v, y and the operators; Tc: compute type (T, or float pairs ff for
-// FP64X with double storage)
-template <typename T, typename Tc>
-__global__ void __launch_bounds__(256)
-hv_simt_sec_kernel(const T* __restrict__ v, T* __restrict__ y, const T* __restrict__ Lsub,
-                   const T* __restrict__ Rsub, SecParams p) {
-  __shared__ Tc As[SBK][SBM];
-  __shared__ Tc Bs[SBK][SBN];
-  const TileD t = p.tiles[blockIdx.x];
-  const RowSegD rs = p.rseg[t.rs];
-  const ColSegD cs = p.cseg[t.cs];
-  const long long base = p.qbase[rs.q];
-  const long long ld = p.qld[rs.q];
-  const int rows = min(SBM, rs.dim - t.r_in), cols = min(SBN, cs.dim - t.c_in);
-  const int r0 = rs.off + t.r_in, c0 = cs.off + t.c_in;
-  const int tid = threadIdx.x, tx = tid % 16, ty = tid / 16;
-  const Tc zero = c_zero<Tc>();
-  Tc acc[4][4];
-#pragma unroll
-  for (int a = 0; a < 4; ++a)
-#pragma unroll
-    for (int b = 0; b < 4; ++b) acc[a][b] = zero;
-  auto mma = [&]() {
-#pragma unroll
-    for (int k = 0; k < SBK; ++k) {
-      Tc av[4], bv[4];
-#pragma unroll
-      for (int a = 0; a < 4; ++a) av[a] = As[k][tx + 16 * a];
-#pragma unroll
-      for (int b = 0; b < 4; ++b) bv[b] = Bs[k][ty + 16 * b];
-#pragma unroll
-      for (int a = 0; a < 4; ++a)
-#pragma unroll
-        for (int b = 0; b < 4; ++b) c_mac(acc[a][b], av[a], bv[b]);
-    }
-  };
-  // phase 1: H_l restricted
-  for (int e = rs.k1b; e < rs.k1e; ++e) {
-    const K1D k = p.k1[e];
-    const T* A = Lsub + k.a_off + (long long)t.r_in * k.kdim;  // A[i][kk] = A[i*kdim + kk]
-    const T* B = v + base + k.b_row + ld * c0;                  // B[kk][j] = B[kk + ld*j]
-    for (int k0 = 0; k0 < k.kdim; k0 += SBK) {
-#pragma unroll
-      for (int r = 0; r < 4; ++r) {
-        const int kk = tid % SBK, i = tid / SBK + 16 * r;
-        const int gk = k0 + kk;
-        As[kk][i] = (i < rows && gk < k.kdim) ? c_in<Tc>(A[(long long)i * k.kdim + gk]) : zero;
-        Bs[kk][i] = (i < cols && gk < k.kdim) ? c_in<Tc>(B[gk + ld * i]) : zero;
-      }
-      __syncthreads();
-      mma();
-      __syncthreads();
-    }
-  }
-  // phase 2: H_r restricted
-  for (int e = cs.k2b; e < cs.k2e; ++e) {
-    const K2D k = p.k2[e];
-    const T* A = v + base + r0 + ld * k.a_col;                  // A[i][kk] = A[i + ld*kk]
-    const T* B = Rsub + k.b_off + (long long)t.c_in * k.kdim;   // B[kk][j] = B[j*kdim + kk]
-    for (int k0 = 0; k0 < k.kdim; k0 += SBK) {
-#pragma unroll
-      for (int r = 0; r < 4; ++r) {
-        const int i = tid % SBM, kk = tid / SBM + 4 * r;
-        const int gk = k0 + kk;
-        As[kk][i] = (i < rows && gk < k.kdim) ? c_in<Tc>(A[i + ld * gk]) : zero;
-        const int kb = tid % SBK, j = tid / SBK + 16 * r;
-        const int gkb = k0 + kb;
-        Bs[kb][j] = (j < cols && gkb < k.kdim) ? c_in<Tc>(B[(long long)j * k.kdim + gkb]) : zero;
-      }
-      __syncthreads();
-      mma();
-      __syncthreads();
-    }
-  }
-  T* Y = y + base + r0 + ld * c0;
-#pragma unroll
-  for (int a = 0; a < 4; ++a)
-#pragma unroll
-    for (int b = 0; b < 4; ++b) {
-      const int i = tx + 16 * a, j = ty + 16 * b;
-      if (i < rows && j < cols) Y[i + ld * j] = c_out(acc[a][b]);
-    }
-  // zero padding rows of the segment (last row tile of the segment only)
-  if (t.r_in + SBM >= rs.dim) {
-    const int npad = rs.dim_pad - rs.dim;
-    for (int q = tid; q < npad * SBN; q += 256) {
-      const int i = q % npad, j = q / npad;
-      if (j < cols) y[base + rs.off + rs.dim + i + ld * (c0 + j)] = T(0);
-    }
-  }
-}
-
-// Four rows of a column as the compute type (p aligned to four elements when VEC).
-template <typename Tout, bool VEC>
-__device__ __forceinline__ void load4(const double* p, Tout (&o)[4]) {
-  if constexpr (VEC) {
-    const double2 a = *(const double2*)p, b = *(const double2*)(p + 2);
-    o[0] = (Tout)a.x, o[1] = (Tout)a.y, o[2] = (Tout)b.x, o[3] = (Tout)b.y;
-  } else {
-#pragma unroll
-    for (int i = 0; i < 4; ++i) o[i] = (Tout)p[i];
-  }
-}
-template <typename Tout, bool VEC>
-__device__ __forceinline__ void load4(const float* p, Tout (&o)[4]) {
-  if constexpr (VEC) {
-    const float4 a = *(const float4*)p;
-    o[0] = (Tout)a.x, o[1] = (Tout)a.y, o[2] = (Tout)a.z, o[3] = (Tout)a.w;
-  } else {
-#pragma unroll
-    for (int i = 0; i < 4; ++i) o[i] = (Tout)p[i];
-  }
-}
-template <typename Tout, bool VEC>
-__device__ __forceinline__ void load4(const __nv_bfloat16* p, Tout (&o)[4]) {
-  if constexpr (VEC) {
-    const uint2 u = *(const uint2*)p;
-    o[0] = (Tout)__uint_as_float(u.x << 16), o[1] = (Tout)__uint_as_float(u.x & 0xffff0000u);
-    o[2] = (Tout)__uint_as_float(u.y << 16), o[3] = (Tout)__uint_as_float(u.y & 0xffff0000u);
-  } else {
-#pragma unroll
-    for (int i = 0; i < 4; ++i) o[i] = (Tout)__bfloat162float(p[i]);
-  }
-}
-
-// Y(sub-block) += sum_moves c * V(source sub-block).  Bound by memory: a thread takes four
-// rows of one column (segments start at multiples of 8 rows, so the fours of an aligned
-// vector are aligned) and walks the block's moves with their addresses precomputed.  The
-// earlier form (one row per thread of 256, eight columns, three dependent table reads per
-// move) left most lanes of a small sector idle: on the 4-leg Heisenberg sectors of m = 1024
-// the whole BF16 H·v went from 958 to 675 us, on the 3-leg Hubbard ones in TF32 from 5.92
-// to 5.33 ms (there the tile configuration with separate moves became the faster one).
-constexpr int MV_THREADS = 128, MV_ITEMS = 1024;  // threads; fours of rows per block
-template <typename Tin, typename Tout, bool VEC>
-__global__ void __launch_bounds__(MV_THREADS)
-k_sec_moves(const Tin* __restrict__ v, Tout* __restrict__ y, SecParams p, int use64) {
-  const MoveItem it = p.mitems[blockIdx.x];
-  for (int t = threadIdx.x; t < it.nquad * it.ncol; t += MV_THREADS) {
-    const int c = it.c_in + t / it.nquad, i = 4 * (t % it.nquad);
-    Tout acc[4], x[4];
-    Tout* Y = y + it.dst + i + (long long)it.ld * c;
-    load4<Tout, VEC>(Y, acc);
-#pragma unroll 4
-    for (int e = it.mb; e < it.me; ++e) {
-      const MoveRec m = p.mrec[e];
-      load4<Tout, VEC>(v + m.src + i + (long long)m.ld * c, x);
-      const Tout f = use64 ? (Tout)m.c64 : (Tout)m.c32;
-#pragma unroll
-      for (int q = 0; q < 4; ++q) acc[q] += f * x[q];
-    }
-#pragma unroll
-    for (int q = 0; q < 4; ++q)
-      if (i + q < it.dim) Y[q] = acc[q];
-  }
-}
-
-template <typename Tin, typename Tout>
-void launch_moves(const SecParams& p, int nm, const Tin* v, Tout* y, int use64, cudaStream_t s) {
-  // vector loads where both vectors start on a 16-byte boundary
-  if ((((uintptr_t)v | (uintptr_t)y) & 15) == 0)
-    k_sec_moves<Tin, Tout, true><<<nm, MV_THREADS, 0, s>>>(v, y, p, use64);
-  else
-    k_sec_moves<Tin, Tout, false><<<nm, MV_THREADS, 0, s>>>(v, y, p, use64);
-}
-
 __global__ void k_zero_pad(double* __restrict__ x, const long long* __restrict__ off,
                            const int* __restrict__ cnt, int n) {
   const int w = blockIdx.x * blockDim.x + threadIdx.x;
@@ -499,18 +286,9 @@ int sec_build(dmrg2d_ops* ops, const dmrg2d_block* L, const dmrg2d_block* R, con
     }
     cs.k2e = (int)S->k2.size();
   }
-  // ---- CUDA-core tiles ----
-  for (int q = 0; q < S->nQ; ++q)
-    for (size_t r = 0; r < S->rseg.size(); ++r) {
-      if (S->rseg[r].q != q) continue;
-      for (int ri = 0; ri < S->rseg[r].dim; ri += SBM)
-        for (size_t c = 0; c < S->cseg.size(); ++c) {
-          if (S->cseg[c].q != q) continue;
-          for (int ci = 0; ci < S->cseg[c].dim; ci += SBN)
-            S->tiles.push_back({(int)r, (int)c, ri, ci});
-        }
-    }
   // ---- scalar moves per destination sub-block ----
+  LongPlan* lp = new LongPlan();
+  ops->lp = lp;
   for (size_t r = 0; r < S->rseg.size(); ++r)
     for (size_t c = 0; c < S->cseg.size(); ++c) {
       if (S->rseg[r].q != S->cseg[c].q) continue;
@@ -532,31 +310,24 @@ int sec_build(dmrg2d_ops* ops, const dmrg2d_block* L, const dmrg2d_block* R, con
       S->mdst.push_back(md);
       const RowSegD& rs = S->rseg[r];
       const ColSegD& cs = S->cseg[c];
-      const long long dst = S->qbase[rs.q] + rs.off + (long long)S->qld[rs.q] * cs.off;
-      const int nquad = rs.dim_pad / 4, step = std::max(1, MV_ITEMS / nquad);
-      for (int ci = 0; ci < cs.dim; ci += step)
-        S->mitems.push_back({dst, S->qld[rs.q], rs.dim, nquad, ci, std::min(step, cs.dim - ci),
-                             md.mb, md.me});
+      lp_add_moves(lp, S->qbase[rs.q] + rs.off + (long long)S->qld[rs.q] * cs.off, S->qld[rs.q],
+                   rs.dim, rs.dim_pad, cs.dim, md.mb, md.me);
     }
   for (const MoveSrc& m : S->msrc) {
     const RowSegD& sr = S->rseg[m.rs];
     const ColSegD& sc = S->cseg[m.cs];
-    S->mrec.push_back({S->qbase[sr.q] + sr.off + (long long)S->qld[sr.q] * sc.off, S->qld[sr.q],
-                       m.c32, m.c64});
+    lp->mrec.push_back({S->qbase[sr.q] + sr.off + (long long)S->qld[sr.q] * sc.off, S->qld[sr.q],
+                        m.c32, m.c64});
   }
-  // ---- two-pass CUDA-core plan ----
-  {
-    LongPlan& lp = S->lplan;
-    for (const ColSegD& c : S->cseg)
-      lp.segs[0].push_back({S->qbase[c.q], S->qld[c.q], S->qld[c.q], c.off, c.dim, c.dim, c.k2b,
-                            c.k2e});
-    for (const K2D& k : S->k2) lp.ks[0].push_back({k.b_off, k.a_col, k.kdim});
-    for (const RowSegD& r : S->rseg)
-      lp.segs[1].push_back({S->qbase[r.q], S->qld[r.q], S->qcols[r.q], r.off, r.dim, r.dim_pad,
-                            r.k1b, r.k1e});
-    for (const K1D& k : S->k1) lp.ks[1].push_back({k.a_off, k.b_row, k.kdim});
-    lp_items(&lp);
-  }
+  // ---- two-pass plan over the same segments ----
+  for (const ColSegD& c : S->cseg)
+    lp->segs[0].push_back({S->qbase[c.q], S->qld[c.q], S->qld[c.q], c.off, c.dim, c.dim, c.k2b,
+                           c.k2e, 0, 0, 0, 0});
+  for (const K2D& k : S->k2) lp->ks[0].push_back({k.b_off, k.a_col, k.kdim});
+  for (const RowSegD& r : S->rseg)
+    lp->segs[1].push_back({S->qbase[r.q], S->qld[r.q], S->qcols[r.q], r.off, r.dim, r.dim_pad,
+                           r.k1b, r.k1e, 0, 0, 0, 0});
+  for (const K1D& k : S->k1) lp->ks[1].push_back({k.a_off, k.b_row, k.kdim});
   ops->flops = flops;
   // ---- upload ----
   std::vector<float> Lc32(Lc.begin(), Lc.end()), Rc32(Rc.begin(), Rc.end());
@@ -564,20 +335,6 @@ int sec_build(dmrg2d_ops* ops, const dmrg2d_block* L, const dmrg2d_block* R, con
   int st = DMRG2D_OK;
 #define SUP(h, dp) \
   if (st == DMRG2D_OK) st = up(S, h, &dp, nb, s)
-  SUP(S->qbase, S->d_qbase);
-  SUP(S->qld, S->d_qld);
-  SUP(S->rseg, S->d_rseg);
-  SUP(S->cseg, S->d_cseg);
-  SUP(S->k1, S->d_k1);
-  SUP(S->k2, S->d_k2);
-  SUP(S->tiles, S->d_tiles);
-  SUP(S->mrec, S->d_mrec);
-  SUP(S->mitems, S->d_mitems);
-  for (int ps = 0; ps < 2; ++ps) {
-    SUP(S->lplan.segs[ps], S->lplan.d_segs[ps]);
-    SUP(S->lplan.ks[ps], S->lplan.d_ks[ps]);
-    SUP(S->lplan.items[ps], S->lplan.d_items[ps]);
-  }
   SUP(Lc, S->d_L64);
   SUP(Lc32, S->d_L32);
   SUP(Rc, S->d_R64);
@@ -588,6 +345,13 @@ int sec_build(dmrg2d_ops* ops, const dmrg2d_block* L, const dmrg2d_block* R, con
   if (st == DMRG2D_OK) {
     cudaError_t e = cudaStreamSynchronize(s);
     if (e != cudaSuccess) st = set_error(DMRG2D_ECUDA, "sector upload: %s", cudaGetErrorString(e));
+  }
+  if (st == DMRG2D_OK) {
+    lp->op64[0] = S->d_R64;
+    lp->op64[1] = S->d_L64;
+    lp->op32[0] = S->d_R32;
+    lp->op32[1] = S->d_L32;
+    st = lp_finalise(ops, lp, s);
   }
   // ---- grouped tensor-core plan over the same segments ----
   if (st == DMRG2D_OK) {
@@ -630,26 +394,24 @@ void sec_release(dmrg2d_ops* ops) {
 int sec_apply(const dmrg2d_ops* ops, const void* v, void* y, int precision, cudaStream_t s) {
   const SecState* S = (const SecState*)ops->sec;
   if (!S) return set_error(DMRG2D_EINVAL, "not a sector-restricted ops object");
-  const SecParams p = S->params();
-  const int nt = (int)S->tiles.size(), nm = (int)S->mitems.size();
-  // timed kernel: the CUDA-core kernel here; the grouped tensor-core launch times itself
+  const LongPlan* lp = ops->lp;
+  // timed kernel: the block products here; the grouped tensor-core launch times itself
   const bool simt =
       precision == DMRG2D_FP64 || precision == DMRG2D_FP32 || precision == DMRG2D_FP64X;
   auto ev = simt ? prof_slot(ops) : std::pair<cudaEvent_t, cudaEvent_t>(nullptr, nullptr);
   if (ev.first) D2_CUDA(cudaEventRecord(ev.first, s));
   if (precision == DMRG2D_FP64 || precision == DMRG2D_FP64X) {
-    // FP64X: the sub-block products in float pairs, the scalar moves in FP64
+    // FP64X: the block products on split operands, the scalar moves in FP64
     if (precision == DMRG2D_FP64)
-      D2_TRY(lp_launch_f64(&S->lplan, (const double*)v, (double*)y, S->d_L64, S->d_R64, s));
-    else if (nt)
-      hv_simt_sec_kernel<double, ff><<<nt, 256, 0, s>>>((const double*)v, (double*)y, S->d_L64,
-                                                        S->d_R64, p);
+      D2_TRY(lp_launch_f64(lp, (const double*)v, (double*)y, s));
+    else
+      D2_TRY(fx_launch(lp, (const double*)v, (double*)y, s));
     if (ev.second) D2_CUDA(cudaEventRecord(ev.second, s));
-    if (nm) launch_moves(p, nm, (const double*)v, (double*)y, 1, s);
+    D2_TRY(lp_moves_f64(lp, (const double*)v, (double*)y, s));
   } else if (precision == DMRG2D_FP32) {
-    D2_TRY(lp_launch_f32(&S->lplan, (const float*)v, (float*)y, S->d_L32, S->d_R32, s));
+    D2_TRY(lp_launch_f32(lp, (const float*)v, (float*)y, s));
     if (ev.second) D2_CUDA(cudaEventRecord(ev.second, s));
-    if (nm) launch_moves(p, nm, (const float*)v, (float*)y, 0, s);
+    D2_TRY(lp_moves_f32(lp, (const float*)v, (float*)y, s));
   } else if (precision == DMRG2D_BF16X3 && S->gp_ok && ops->tc_cfg[DMRG2D_BF16] == 2 * gp_num_configs()) {
     // segment kernels: three products, then the moves on v_hi and v_lo
     const __nv_bfloat16* vhi = (const __nv_bfloat16*)v;
@@ -657,19 +419,17 @@ int sec_apply(const dmrg2d_ops* ops, const void* v, void* y, int precision, cuda
     D2_TRY(gp_launch_seg(ops, &S->plan, vhi, (float*)y, DMRG2D_BF16, s, false, false));
     D2_TRY(gp_launch_seg(ops, &S->plan, vlo, (float*)y, DMRG2D_BF16, s, false, true));
     D2_TRY(gp_launch_seg(ops, &S->plan, vhi, (float*)y, DMRG2D_BF16, s, true, true));
-    if (nm) {
-      launch_moves(p, nm, vhi, (float*)y, 0, s);
-      launch_moves(p, nm, vlo, (float*)y, 0, s);
-    }
+    D2_TRY(lp_moves_bf16(lp, vhi, (float*)y, s));
+    D2_TRY(lp_moves_bf16(lp, vlo, (float*)y, s));
   } else if ((precision == DMRG2D_TF32 || precision == DMRG2D_BF16) && S->gp_ok &&
              ops->tc_cfg[precision] == 2 * gp_num_configs()) {
     // segment kernels (M along the long dimension of each V_q), then the scalar moves
     D2_TRY(gp_launch_seg(ops, &S->plan, v, (float*)y, precision, s));
-    if (nm) {
+    {
       if (precision == DMRG2D_BF16)
-        launch_moves(p, nm, (const __nv_bfloat16*)v, (float*)y, 0, s);
+        D2_TRY(lp_moves_bf16(lp, (const __nv_bfloat16*)v, (float*)y, s));
       else
-        launch_moves(p, nm, (const float*)v, (float*)y, 0, s);
+        D2_TRY(lp_moves_f32(lp, (const float*)v, (float*)y, s));
     }
   } else if (precision == DMRG2D_BF16X3 && S->gp_ok) {
     // v = [v_hi | v_lo]: H_hi v_hi + H_hi v_lo + H_lo v_hi with the layout chosen for BF16,
@@ -681,9 +441,9 @@ int sec_apply(const dmrg2d_ops* ops, const void* v, void* y, int precision, cuda
     D2_TRY(gp_launch(ops, &S->plan, vhi, (float*)y, DMRG2D_BF16, cfg % G, s, fused, false, false));
     D2_TRY(gp_launch(ops, &S->plan, vlo, (float*)y, DMRG2D_BF16, cfg % G, s, fused, false, true));
     D2_TRY(gp_launch(ops, &S->plan, vhi, (float*)y, DMRG2D_BF16, cfg % G, s, false, true, true));
-    if (!fused && nm) {
-      launch_moves(p, nm, vhi, (float*)y, 0, s);
-      launch_moves(p, nm, vlo, (float*)y, 0, s);
+    if (!fused) {
+      D2_TRY(lp_moves_bf16(lp, vhi, (float*)y, s));
+      D2_TRY(lp_moves_bf16(lp, vlo, (float*)y, s));
     }
   } else if ((precision == DMRG2D_TF32 || precision == DMRG2D_BF16) && S->gp_ok) {
     // tc_cfg < G: one launch, the grouped kernel's epilogue adds the scalar moves;
@@ -691,11 +451,11 @@ int sec_apply(const dmrg2d_ops* ops, const void* v, void* y, int precision, cuda
     const int G = gp_num_configs(), cfg = ops->tc_cfg[precision];
     const bool fused = cfg < G;
     D2_TRY(gp_launch(ops, &S->plan, v, (float*)y, precision, cfg % G, s, fused));
-    if (!fused && nm) {
+    if (!fused) {
       if (precision == DMRG2D_BF16)
-        launch_moves(p, nm, (const __nv_bfloat16*)v, (float*)y, 0, s);
+        D2_TRY(lp_moves_bf16(lp, (const __nv_bfloat16*)v, (float*)y, s));
       else
-        launch_moves(p, nm, (const float*)v, (float*)y, 0, s);
+        D2_TRY(lp_moves_f32(lp, (const float*)v, (float*)y, s));
     }
   } else {
     return set_error(DMRG2D_EUNSUPPORTED,

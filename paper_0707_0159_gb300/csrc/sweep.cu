@@ -488,7 +488,7 @@ class Sweeper {
       if (mixed) {
         so.precision = o_.precision;
         so.refine = 1;
-        so.refine_precision = DMRG2D_FP64X;  // outer-loop residuals in float pairs
+        so.refine_precision = DMRG2D_FP64X;  // outer-loop residuals on split operands
         so.inner_iter = std::min(o_.max_iter, 300);
         so.outer_max = 40;
       } else {
