@@ -7,6 +7,8 @@
 //   2. V H_r^T:  for every block (i3, i3') of H_r:  acc += V_tile(i2, i3') * HR[i3,i3']^T
 //   3. scalar moves (H_c and off-diagonal column terms): acc += c * V_tile(i2', i3')
 // and writes Y once.  V is column-major with leading dimension m1*d.
+#include <algorithm>
+
 #include "common.h"
 #include "longplan.h"
 
@@ -25,7 +27,7 @@ struct SimtParams {
   const int* Csrc;
 };
 
-constexpr int BM = 64, BN = 64, BK = 16, TX = 16, TY = 16;  // 256 threads, 4x4 outputs each
+constexpr int BM = 64, BK = 16, TX = 16, TY = 16;  // 256 threads, 4x4 outputs each
 
 // BMt x BNt piece per CTA (64 x 64: 4 x 4 outputs per thread; smaller pieces for small
 // superblocks, whose 64 x 64 grid would leave most SMs idle at GB300's FP64 rate)
@@ -156,6 +158,88 @@ hv_simt_kernel(const T* __restrict__ v, T* __restrict__ y, const T* __restrict__
     }
 }
 
+// Small pieces (TS x TS, one output per thread) for superblocks whose larger pieces leave SMs
+// idle.  The next K chunk of 16 travels through registers while the current one is
+// multiplied; the three phases form one sequence of chunks.  Bound by the FP64 pipe once
+// every SM has the same number of pieces: on the 2-leg m = 64 superblock (V 256 x 256) 16 x
+// 16 pieces without the prefetch took 66 us (256 pieces on 152 SMs: two on most, one on some),
+// 8 x 8 pieces (1024: 6.7 per SM, seven on the fullest) take 47 us; 41 us is the pipe's rate.
+template <typename T, int TS>
+__global__ void __launch_bounds__(TS * TS)
+hv_simt_small_kernel(const T* __restrict__ v, T* __restrict__ y, const T* __restrict__ HL,
+                     const T* __restrict__ HR, const T* __restrict__ Cval, SimtParams p) {
+  constexpr int NT = TS * TS, R = BK * TS / NT;  // elements of each operand per thread
+  __shared__ T As[BK][TS + 1];
+  __shared__ T Bs[BK][TS + 1];
+  const int m1 = p.m1, m4 = p.m4;
+  const int nbm = (m1 + TS - 1) / TS, nbn = (m4 + TS - 1) / TS;
+  const int i0 = (blockIdx.x % nbm) * TS, i2 = blockIdx.x / nbm;
+  const int j0 = (blockIdx.y % nbn) * TS, i3 = blockIdx.y / nbn;
+  const int64_t ld = p.ld;
+  const int tid = threadIdx.x, tx = tid % TS, ty = tid / TS;
+  const int kk = tid % BK, kr = tid / BK;  // K and row of k-contiguous operands
+  const int nL = p.Lptr[i2 + 1] - p.Lptr[i2], nR = p.Rptr[i3 + 1] - p.Rptr[i3];
+  T ra[R], rb[R];
+  auto fetch = [&](int e, int k0) {  // chunk k0 of block e (H_l blocks first)
+    if (e < nL) {
+      const int g = p.Lptr[i2] + e;
+      const T* A = HL + (size_t)g * m1 * m1;
+      const T* B = v + (int64_t)p.Lcol[g] * m1 + ld * ((int64_t)i3 * m4);
+#pragma unroll
+      for (int r = 0; r < R; ++r) {
+        const int q = kr + r * (NT / BK);
+        const bool in = k0 + kk < m1;
+        ra[r] = in && i0 + q < m1 ? A[(size_t)(i0 + q) * m1 + k0 + kk] : T(0);
+        rb[r] = in && j0 + q < m4 ? B[k0 + kk + ld * (j0 + q)] : T(0);
+      }
+    } else {
+      const int g = p.Rptr[i3] + e - nL;
+      const T* A = v + (int64_t)i2 * m1 + ld * ((int64_t)p.Rcol[g] * m4);
+      const T* B = HR + (size_t)g * m4 * m4;
+#pragma unroll
+      for (int r = 0; r < R; ++r) {
+        const int k = ty + r * TS, q = kr + r * (NT / BK);
+        ra[r] = k0 + k < m4 && i0 + tx < m1 ? A[i0 + tx + ld * (k0 + k)] : T(0);
+        rb[r] = k0 + kk < m4 && j0 + q < m4 ? B[(size_t)(j0 + q) * m4 + k0 + kk] : T(0);
+      }
+    }
+  };
+  T acc = T(0);
+  int e = 0, k0 = 0;
+  if (nL + nR > 0) fetch(0, 0);
+  while (e < nL + nR) {
+    __syncthreads();
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+      const int q = kr + r * (NT / BK);
+      if (e < nL)
+        As[kk][q] = ra[r];
+      else
+        As[ty + r * TS][tx] = ra[r];
+      Bs[kk][q] = rb[r];
+    }
+    __syncthreads();
+    k0 += BK;
+    if (k0 >= (e < nL ? m1 : m4)) {
+      k0 = 0;
+      ++e;
+    }
+    if (e < nL + nR) fetch(e, k0);
+#pragma unroll
+    for (int k = 0; k < BK; ++k) acc += As[k][tx] * Bs[k][ty];
+  }
+  const int gi = i0 + tx, gj = j0 + ty;
+  if (gi >= m1 || gj >= m4) return;
+  const int t = i2 + p.d * i3;
+  for (int c = p.Cptr[t]; c < p.Cptr[t + 1]; ++c) {
+    const int src = p.Csrc[c];
+    acc += Cval[c] * v[(int64_t)(src % p.d) * m1 + gi + ld * ((int64_t)(src / p.d) * m4 + gj)];
+  }
+  y[(int64_t)i2 * m1 + gi + ld * ((int64_t)i3 * m4 + gj)] = acc;
+}
+
+int sm_count(const dmrg2d_ops* ops) { return ops->lp ? ops->lp->sms : 1; }
+
 template <typename T>
 int launch(const dmrg2d_ops* ops, const T* v, T* y, const T* HL, const T* HR, const T* C,
            cudaStream_t s) {
@@ -170,31 +254,59 @@ int launch(const dmrg2d_ops* ops, const T* v, T* y, const T* HL, const T* HR, co
   p.Rcol = ops->dev.Rcol;
   p.Cptr = ops->dev.Cptr;
   p.Csrc = ops->dev.Csrc;
-  // the largest piece (64, 32 or 16 square) whose grid still gives every SM a CTA
-  static int sms = 0;
-  if (!sms) {
-    int dev = 0;
-    cudaGetDevice(&dev);
-    if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) sms = 1;
-  }
-  auto ctas = [&](int b) {
-    return ((int64_t)(ops->m1 + b - 1) / b) * ops->d * ((int64_t)(ops->m4 + b - 1) / b) * ops->d;
+  const int sms = sm_count(ops);
+  auto ctas = [&](int64_t b) {
+    return ((ops->m1 + b - 1) / b) * ops->d * ((ops->m4 + b - 1) / b) * ops->d;
   };
-  const int tb = ctas(64) >= sms ? 64 : (ctas(32) >= sms ? 32 : 16);
+  int tb;
+  bool two_pass = false;
+  if (sizeof(T) == 8) {
+    // Every kernel runs at the FP64 pipe's rate, so the time is the fullest SM's outputs times
+    // their padded K: pieces of 64, 32, 16 or 8, or the two-pass kernel, which pads nothing
+    // but takes two kernels more and 1.1 of the rate, once it has two items per SM.
+    // (3-leg Heisenberg 250 x 131: pieces of 64 9.63 ms, two-pass 6.13 ms; 2-leg 200 x 200:
+    // pieces of 64 2.53 ms, of 8 1.31 ms; 2-leg Hubbard 40 x 40: 0.99 and 0.34 ms.)
+    auto pad = [](int m, int64_t b) { return (double)((m + b - 1) / b * b) / m; };
+    double best = 0.0;
+    tb = 0;
+    for (int b : {64, 32, 16, 8}) {
+      const int64_t g = ctas(b);
+      const double kpad = std::max(pad(ops->m1, BK), pad(ops->m4, BK));
+      const double cost = (double)((g + sms - 1) / sms) * b * b * kpad;
+      if (!tb || cost < 0.98 * best) {
+        best = cost;
+        tb = b;
+      }
+    }
+    two_pass = (int)ops->lp->items[0].size() >= 2 * sms &&
+               1.1 * (double)ops->n_vec / sms < 0.98 * best;
+  } else {
+    // the largest piece (64, 32 or 16 square) whose grid still gives every SM a CTA
+    tb = ctas(64) >= sms ? 64 : (ctas(32) >= sms ? 32 : 16);
+  }
   const int64_t gx = (int64_t)((ops->m1 + tb - 1) / tb) * ops->d;
   const int64_t gy = (int64_t)((ops->m4 + tb - 1) / tb) * ops->d;
-  if (gx > 0x7fffffff || gy > 65535)
+  if (!two_pass && (gx > 0x7fffffff || gy > 65535))
     return set_error(DMRG2D_EUNSUPPORTED, "SIMT grid %lld x %lld too large", (long long)gx,
                      (long long)gy);
   dim3 grid((unsigned)gx, (unsigned)gy);
   auto ev = prof_slot(ops);
   if (ev.first) D2_CUDA(cudaEventRecord(ev.first, s));
+  if constexpr (sizeof(T) == 8) {
+    if (two_pass) {
+      D2_TRY(lp_launch_f64(ops->lp, v, y, s));
+      if (ev.second) D2_CUDA(cudaEventRecord(ev.second, s));
+      return lp_moves_f64(ops->lp, v, y, s);
+    }
+  }
   if (tb == 64)
     hv_simt_kernel<T, 64, 64><<<grid, TX * TY, 0, s>>>(v, y, HL, HR, C, p);
   else if (tb == 32)
     hv_simt_kernel<T, 32, 32><<<grid, TX * TY, 0, s>>>(v, y, HL, HR, C, p);
+  else if (tb == 16)
+    hv_simt_small_kernel<T, 16><<<grid, 256, 0, s>>>(v, y, HL, HR, C, p);
   else
-    hv_simt_kernel<T, 16, 16><<<grid, TX * TY, 0, s>>>(v, y, HL, HR, C, p);
+    hv_simt_small_kernel<T, 8><<<grid, 64, 0, s>>>(v, y, HL, HR, C, p);
   D2_CUDA(cudaGetLastError());
   if (ev.second) D2_CUDA(cudaEventRecord(ev.second, s));
   return DMRG2D_OK;
