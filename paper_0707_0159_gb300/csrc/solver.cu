@@ -16,7 +16,10 @@
 #include <algorithm>
 #include <chrono>
 #include <cmath>
+#include <mutex>
 #include <vector>
+
+#include <cooperative_groups.h>
 
 #include "common.h"
 
@@ -116,6 +119,119 @@ __global__ void k_lz_axpy2(double* __restrict__ w, const double* __restrict__ qj
     if (qjm1) r -= b * qjm1[e];
     w[e] = r;
   }
+}
+
+// ---- one Lanczos step's vector work in one kernel -------------------------------------
+// alpha_j = q_j . w; w -= alpha_j q_j + beta_{j-1} q_{j-1}; `passes` Gram-Schmidt passes
+// against q_0 .. q_j; beta_j = |w|; q_{j+1} = w / beta_j.  For vectors that fit in the SMs'
+// shared memory: every CTA keeps its part of w there, and the four reductions over the grid
+// are grid barriers of one cooperative launch (each CTA then adds the partial sums of all
+// CTAs in the same order).  As separate kernels the step was twelve launches of a few
+// microseconds each: 124 us next to an H·v of 66 us on the 2-leg m = 64 superblock (n = 65536,
+// 40 steps); in one kernel 48 us.
+// The FP64 pipe (2 operations per clock and SM) makes every redundant addition count: sums
+// over a CTA or the grid are finished by one warp.
+constexpr int LZ_T = 512, LZ_CHUNK = 5120;  // threads; vector elements per CTA at most
+
+// v summed over the CTA; valid in thread 0
+__device__ double lz_block_sum(double v, double* red) {
+  v = warp_sum(v);
+  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = v;
+  __syncthreads();
+  double r = 0.0;
+  if (threadIdx.x < 32) {
+    r = threadIdx.x < LZ_T / 32 ? red[threadIdx.x] : 0.0;
+#pragma unroll
+    for (int o = LZ_T / 64; o > 0; o >>= 1) r += __shfl_down_sync(0xffffffffu, r, o);
+  }
+  return r;
+}
+// the sum of the grid's partial sums, in every thread
+__device__ double lz_grid_sum(const double* part, double* red) {
+  if (threadIdx.x < 32) {
+    double v = 0.0;
+    for (int i = threadIdx.x; i < gridDim.x; i += 32) v += __ldcg(part + i);
+    v = warp_sum(v);
+    if (threadIdx.x == 0) red[0] = v;
+  }
+  __syncthreads();
+  const double r = red[0];
+  __syncthreads();
+  return r;
+}
+
+__global__ void __launch_bounds__(LZ_T)
+k_lz_step(double* __restrict__ Q, int64_t n, int j, const double* __restrict__ w,
+          double* __restrict__ alpha, double* __restrict__ beta, double* part, int passes,
+          int chunk) {
+  extern __shared__ double ws[];  // chunk of w, then h[0..j]
+  __shared__ double red[LZ_T / 32];
+  double* hs = ws + chunk;
+  const cooperative_groups::grid_group grid = cooperative_groups::this_grid();
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, G = gridDim.x;
+  const int64_t base = (int64_t)blockIdx.x * chunk;
+  const int len = (int)max((int64_t)0, min((int64_t)chunk, n - base));
+  const double* Qb = Q + base;
+  const double* qj = Qb + (int64_t)j * n;
+  double s = 0.0;
+  for (int e = tid; e < len; e += LZ_T) {
+    const double we = w[base + e];
+    ws[e] = we;
+    s += qj[e] * we;
+  }
+  s = lz_block_sum(s, red);
+  if (tid == 0) part[blockIdx.x] = s;
+  grid.sync();
+  const double a = lz_grid_sum(part, red);
+  part += G;
+  if (blockIdx.x == 0 && tid == 0) alpha[j] = a;
+  const double b = j > 0 ? beta[j - 1] : 0.0;
+  for (int e = tid; e < len; e += LZ_T) {
+    double r = ws[e] - a * qj[e];
+    if (j > 0) r -= b * (qj - n)[e];
+    ws[e] = r;
+  }
+  for (int pass = 0; pass < passes; ++pass) {
+    __syncthreads();
+    for (int k = warp; k <= j; k += LZ_T / 32) {  // a warp per basis vector
+      const double* qk = Qb + (int64_t)k * n;
+      double d0 = 0.0, d1 = 0.0;
+      int e = lane;
+#pragma unroll 2
+      for (; e + 32 < len; e += 64) {
+        d0 += qk[e] * ws[e];
+        d1 += qk[e + 32] * ws[e + 32];
+      }
+      if (e < len) d0 += qk[e] * ws[e];
+      d0 = warp_sum(d0 + d1);
+      if (lane == 0) part[(int64_t)k * G + blockIdx.x] = d0;
+    }
+    grid.sync();
+    for (int k = warp; k <= j; k += LZ_T / 32) {
+      double d = 0.0;
+      for (int i = lane; i < G; i += 32) d += __ldcg(part + (int64_t)k * G + i);
+      d = warp_sum(d);
+      if (lane == 0) hs[k] = d;
+    }
+    part += (int64_t)(j + 1) * G;
+    __syncthreads();
+    for (int e = tid; e < len; e += LZ_T) {
+      double d = 0.0;
+#pragma unroll 4
+      for (int k = 0; k <= j; ++k) d += hs[k] * Qb[(int64_t)k * n + e];
+      ws[e] -= d;
+    }
+  }
+  s = 0.0;
+  for (int e = tid; e < len; e += LZ_T) s += ws[e] * ws[e];
+  s = lz_block_sum(s, red);
+  if (tid == 0) part[blockIdx.x] = s;
+  grid.sync();
+  const double nrm = sqrt(lz_grid_sum(part, red));
+  if (blockIdx.x == 0 && tid == 0) beta[j] = nrm;
+  const double f = nrm > 0.0 ? 1.0 / nrm : 0.0;
+  double* qn = Q + base + (int64_t)(j + 1) * n;
+  for (int e = tid; e < len; e += LZ_T) qn[e] = ws[e] * f;
 }
 
 // out = in / *nrm   (zero when the norm is zero)
@@ -1186,6 +1302,24 @@ struct Ctx {
     D2_CUDA(cudaGetLastError());
     return DMRG2D_OK;
   }
+  // CTAs of k_lz_step for this vector length; 0 when it does not fit (or no cooperative launch)
+  int lz_grid() const {
+    int dev = 0, sms = 0, coop = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess ||
+        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
+        cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev) != cudaSuccess || !coop)
+      return 0;
+    if (n > (int64_t)sms * LZ_CHUNK) return 0;
+    return (int)std::max<int64_t>(1, std::min<int64_t>(sms, (n + 127) / 128));
+  }
+  int lz_step(double* Q, int j, const double* w, double* alpha, double* beta, int passes, int grid) {
+    int chunk = (int)((n + grid - 1) / grid);
+    int64_t len = n;
+    void* args[] = {&Q, &len, &j, &w, &alpha, &beta, &part, &passes, &chunk};
+    D2_CUDA(cudaLaunchCooperativeKernel((const void*)k_lz_step, dim3(grid), dim3(LZ_T), args,
+                                        sizeof(double) * (chunk + j + 1), s));
+    return DMRG2D_OK;
+  }
   // read k device doubles into the pinned mirror and wait
   int fetch(const double* dsrc, int k) {
     D2_CUDA(cudaMemcpyAsync(hscal, dsrc, k * sizeof(double), cudaMemcpyDeviceToHost, s));
@@ -1203,6 +1337,73 @@ int dmalloc(DevBuf& b, size_t bytes) {
   return DMRG2D_OK;
 }
 
+// 64 pinned doubles for the scalars a solve reads back.  cudaMallocHost and cudaFreeHost took
+// 270 us of every call (a quarter of the first Lanczos steps of a small superblock), so up to
+// PINNED_KEPT slots are kept between calls: one per solve running at a time, under a mutex,
+// given back after the solve's stream has finished.
+constexpr int PINNED_KEPT = 8;
+struct PinnedSlot {
+  double* p = nullptr;
+  cudaStream_t s = nullptr;
+  static std::vector<double*>& kept() {
+    static std::vector<double*> v;
+    return v;
+  }
+  static std::mutex& mu() {
+    static std::mutex m;
+    return m;
+  }
+  int take(cudaStream_t stream) {
+    s = stream;
+    {
+      std::lock_guard<std::mutex> lk(mu());
+      if (!kept().empty()) {
+        p = kept().back();
+        kept().pop_back();
+      }
+    }
+    if (p) {  // still pinned (the device may have been reset meanwhile)?
+      cudaPointerAttributes a;
+      if (cudaPointerGetAttributes(&a, p) == cudaSuccess && a.type == cudaMemoryTypeHost)
+        return DMRG2D_OK;
+      cudaGetLastError();
+      p = nullptr;
+    }
+    D2_CUDA(cudaHostAlloc((void**)&p, sizeof(double) * 64, cudaHostAllocPortable));
+    return DMRG2D_OK;
+  }
+  ~PinnedSlot() {
+    if (!p) return;
+    const bool idle = cudaStreamSynchronize(s) == cudaSuccess;  // no copy into it is in flight
+    if (idle) {
+      std::lock_guard<std::mutex> lk(mu());
+      if ((int)kept().size() < PINNED_KEPT) {
+        kept().push_back(p);
+        return;
+      }
+    }
+    cudaFreeHost(p);
+  }
+};
+
+// Several device buffers in one allocation (each on a 256-byte boundary): cudaMalloc and
+// cudaFree cost tens of microseconds each, cudaFree a wait for the device too.
+struct Part {
+  void* p;  // address of the pointer that receives the buffer
+  size_t bytes;
+};
+int carve(DevBuf& b, std::initializer_list<Part> parts) {
+  size_t total = 0;
+  for (const Part& q : parts) total += (q.bytes + 255) / 256 * 256;
+  D2_TRY(dmalloc(b, total));
+  char* at = (char*)b.p;
+  for (const Part& q : parts) {
+    *(void**)q.p = at;
+    at += (q.bytes + 255) / 256 * 256;
+  }
+  return DMRG2D_OK;
+}
+
 // Lanczos from x (FP64, any norm); on return x holds the normalised Ritz vector.
 // scal layout: [0] theta, [1] resid, [2] status, [3..] scratch scalars
 int lanczos(Ctx& C, int prec, double* x, int max_iter, int kdim, double tol, int fixed,
@@ -1213,26 +1414,20 @@ int lanczos(Ctx& C, int prec, double* x, int max_iter, int kdim, double tol, int
   if (kdim > max_iter + 1) kdim = max_iter + 1;
   if (thick_keep > TR_KEEP_MAX) thick_keep = TR_KEEP_MAX;
   if (thick_keep > kdim - 1) thick_keep = kdim - 1;
-  DevBuf Qb, wb, ab, bb, hb, sb, tb, Mb, rb;
-  if (thick_keep > 0) {
-    D2_TRY(dmalloc(Mb, sizeof(double) * (size_t)(kdim + 1) * thick_keep));
-    D2_TRY(dmalloc(rb, sizeof(double) * (size_t)thick_keep * (6 * (kdim + 1) + thick_keep)));
-  }
-  D2_TRY(dmalloc(Qb, sizeof(double) * (size_t)(kdim + 1) * n));
-  D2_TRY(dmalloc(wb, sizeof(double) * n));
-  D2_TRY(dmalloc(ab, sizeof(double) * (kdim + 1)));
-  D2_TRY(dmalloc(bb, sizeof(double) * (kdim + 1)));
-  D2_TRY(dmalloc(hb, sizeof(double) * (kdim + 1)));
-  D2_TRY(dmalloc(sb, sizeof(double) * (kdim + 1)));
-  D2_TRY(dmalloc(tb, sizeof(double) * 6 * (kdim + 1)));
-  double* Q = (double*)Qb.p;
-  double* w = (double*)wb.p;
-  double* alpha = (double*)ab.p;
-  double* beta = (double*)bb.p;
-  double* h = (double*)hb.p;
-  double* sv = (double*)sb.p;
-  double* scr = (double*)tb.p;
+  DevBuf buf;
+  double *Q, *w, *alpha, *beta, *h, *sv, *scr, *Mk, *rk;
+  const size_t kd = sizeof(double) * (kdim + 1), tk = thick_keep;
+  D2_TRY(carve(buf, {{&Q, kd * n},
+                     {&w, sizeof(double) * n},
+                     {&alpha, kd},
+                     {&beta, kd},
+                     {&h, kd},
+                     {&sv, kd},
+                     {&scr, 6 * kd},
+                     {&Mk, tk * kd},
+                     {&rk, tk * (6 * kd + sizeof(double) * tk)}}));
   double* out3 = C.scal;
+  const int lz_grid = C.lz_grid();
 
   D2_TRY(C.nrm(x, C.scal + 3));
   D2_TRY(C.scale_inv(Q, x, C.scal + 3));
@@ -1243,15 +1438,19 @@ int lanczos(Ctx& C, int prec, double* x, int max_iter, int kdim, double tol, int
   while (true) {
     double* qj = Q + (int64_t)j * n;
     D2_TRY(C.hv(prec, qj, w));
-    D2_TRY(C.dot(qj, w, alpha + j));
-    k_lz_axpy2<<<vgrid(n), VT, 0, C.s>>>(w, qj, j > 0 ? qj - n : nullptr, alpha + j,
-                                        j > 0 ? beta + j - 1 : nullptr, n);
-    D2_CUDA(cudaGetLastError());
-    for (int pass = 0; pass < gs_passes; ++pass) {  // CGS2 (or fewer) against q_0..q_j
-      D2_TRY(C.multidot(Q, n, j + 1, w, h));
-      D2_TRY(C.combo(w, Q, n, j + 1, h, -1));
+    if (lz_grid > 0) {  // leaves q_{j+1} = w / beta_j in the basis
+      D2_TRY(C.lz_step(Q, j, w, alpha, beta, gs_passes, lz_grid));
+    } else {
+      D2_TRY(C.dot(qj, w, alpha + j));
+      k_lz_axpy2<<<vgrid(n), VT, 0, C.s>>>(w, qj, j > 0 ? qj - n : nullptr, alpha + j,
+                                          j > 0 ? beta + j - 1 : nullptr, n);
+      D2_CUDA(cudaGetLastError());
+      for (int pass = 0; pass < gs_passes; ++pass) {  // CGS2 (or fewer) against q_0..q_j
+        D2_TRY(C.multidot(Q, n, j + 1, w, h));
+        D2_TRY(C.combo(w, Q, n, j + 1, h, -1));
+      }
+      D2_TRY(C.nrm(w, beta + j));
     }
-    D2_TRY(C.nrm(w, beta + j));
     ++j;
     ++total;
     const bool last = total >= max_iter;
@@ -1269,14 +1468,13 @@ int lanczos(Ctx& C, int prec, double* x, int max_iter, int kdim, double tol, int
       const bool conv = !fixed && resid <= tol * fabs(theta);
       if (full && !conv && !last && thick_keep > 0) {
         // thick restart: q_j = w / beta_{j-1} joins the re-tridiagonalised Ritz space
-        D2_TRY(C.scale_inv(Q + (int64_t)j * n, w, beta + j - 1));
-        k_thick_restart<<<1, TD_THREADS, 0, C.s>>>(alpha, beta, j, thick_keep, (double*)Mb.p,
-                                                   (double*)rb.p, C.scal + 7);
+        if (lz_grid == 0) D2_TRY(C.scale_inv(Q + (int64_t)j * n, w, beta + j - 1));
+        k_thick_restart<<<1, TD_THREADS, 0, C.s>>>(alpha, beta, j, thick_keep, Mk, rk, C.scal + 7);
         D2_CUDA(cudaGetLastError());
         D2_TRY(C.fetch(C.scal + 7, 1));
         const int pk = (int)C.hscal[0];
         if (pk >= 1) {
-          k_combo_multi<<<vgrid(n), VT, 0, C.s>>>(Q, n, j, (const double*)Mb.p, pk, n);
+          k_combo_multi<<<vgrid(n), VT, 0, C.s>>>(Q, n, j, Mk, pk, n);
           D2_CUDA(cudaGetLastError());
           D2_CUDA(cudaMemcpyAsync(Q + (int64_t)pk * n, Q + (int64_t)j * n, sizeof(double) * n,
                                   cudaMemcpyDeviceToDevice, C.s));
@@ -1302,7 +1500,7 @@ int lanczos(Ctx& C, int prec, double* x, int max_iter, int kdim, double tol, int
         continue;
       }
     }
-    D2_TRY(C.scale_inv(Q + (int64_t)j * n, w, beta + j - 1));
+    if (lz_grid == 0) D2_TRY(C.scale_inv(Q + (int64_t)j * n, w, beta + j - 1));
   }
   D2_TRY(C.nrm(x, C.scal + 3));
   D2_TRY(C.scale_inv(x, x, C.scal + 3));
@@ -1322,20 +1520,17 @@ int lanczos_lo(Ctx& C, int prec, double* x, int max_iter, int kdim, double tol, 
   const int64_t n = C.n;
   if (kdim < 2) kdim = 2;
   if (kdim > max_iter + 1) kdim = max_iter + 1;
-  DevBuf Qb, ab, bb, hb, sb, tb;
-  D2_TRY(dmalloc(Qb, sizeof(float) * (size_t)(kdim + 1) * n));
-  D2_TRY(dmalloc(ab, sizeof(double) * (kdim + 1)));
-  D2_TRY(dmalloc(bb, sizeof(double) * (kdim + 1)));
-  D2_TRY(dmalloc(hb, sizeof(double) * (kdim + 1)));
-  D2_TRY(dmalloc(sb, sizeof(double) * (kdim + 1)));
-  D2_TRY(dmalloc(tb, sizeof(double) * 6 * (kdim + 1)));
-  float* Q = (float*)Qb.p;
+  DevBuf buf;
+  float* Q;
+  double *alpha, *beta, *h, *sv, *scr;
+  const size_t kd = sizeof(double) * (kdim + 1);
+  D2_TRY(carve(buf, {{&Q, sizeof(float) * (size_t)(kdim + 1) * n},
+                     {&alpha, kd},
+                     {&beta, kd},
+                     {&h, kd},
+                     {&sv, kd},
+                     {&scr, 6 * kd}}));
   float* w = C.y32;  // H~ q_j lands here and is orthogonalised in place
-  double* alpha = (double*)ab.p;
-  double* beta = (double*)bb.p;
-  double* h = (double*)hb.p;
-  double* sv = (double*)sb.p;
-  double* scr = (double*)tb.p;
   double* out3 = C.scal;
   const int g = vgrid(n);
   auto start_from_x = [&]() -> int {
@@ -1476,23 +1671,22 @@ static int mixed_outer(Ctx& C, const dmrg2d_solver_opts* o, double* x, double* e
   const int64_t n = C.n;
   const int prec = o->precision;
   const int smax = 6;
-  DevBuf Ub, Wb, hxb, rb, tb, r32b, x32b, t32b, p32b, Gb, cb, scb;
-  D2_TRY(dmalloc(Ub, sizeof(double) * (size_t)smax * n));
-  D2_TRY(dmalloc(Wb, sizeof(double) * (size_t)smax * n));
-  D2_TRY(dmalloc(hxb, sizeof(double) * n));
-  D2_TRY(dmalloc(rb, sizeof(double) * n));
-  D2_TRY(dmalloc(tb, sizeof(double) * n));
-  D2_TRY(dmalloc(r32b, sizeof(float) * n));  // the CG's vectors, FP32
-  D2_TRY(dmalloc(x32b, sizeof(float) * n));
-  D2_TRY(dmalloc(t32b, sizeof(float) * n));
-  D2_TRY(dmalloc(p32b, sizeof(float) * n));
-  D2_TRY(dmalloc(Gb, sizeof(double) * smax * smax));
-  D2_TRY(dmalloc(cb, sizeof(double) * smax));
-  D2_TRY(dmalloc(scb, sizeof(double) * 2 * smax * smax));
-  double *U = (double*)Ub.p, *W = (double*)Wb.p, *hx = (double*)hxb.p, *r = (double*)rb.p;
-  double *t = (double*)tb.p, *G = (double*)Gb.p;
-  float *r32 = (float*)r32b.p, *x32 = (float*)x32b.p, *t32 = (float*)t32b.p, *p32 = (float*)p32b.p;
-  double *cc = (double*)cb.p, *scr = (double*)scb.p;
+  DevBuf buf;
+  double *U, *W, *hx, *r, *t, *G, *cc, *scr;
+  float *r32, *x32, *t32, *p32;  // the CG's vectors, FP32
+  const size_t vd = sizeof(double) * n, vf = sizeof(float) * n, gd = sizeof(double) * smax;
+  D2_TRY(carve(buf, {{&U, smax * vd},
+                     {&W, smax * vd},
+                     {&hx, vd},
+                     {&r, vd},
+                     {&t, vd},
+                     {&r32, vf},
+                     {&x32, vf},
+                     {&t32, vf},
+                     {&p32, vf},
+                     {&G, gd * smax},
+                     {&cc, gd},
+                     {&scr, 2 * gd * smax}}));
   double* sc = C.scal;  // scalars: [4] tmp dot, [5..] host-fetched, [CG_XQ..] CG state
   const int g = vgrid(n);
   StepGraph step;  // the inner CG step, captured once and replayed
@@ -1637,22 +1831,15 @@ extern "C" int dmrg2d_lanczos_ground(const dmrg2d_ops* ops, const dmrg2d_solver_
   C.s = (cudaStream_t)stream;
   C.n = ops->n_vec;
   C.st = &local;
-  DevBuf part, scal, lo, y32;
-  D2_TRY(dmalloc(part, sizeof(double) * (size_t)RED_BLOCKS * 520));
-  D2_TRY(dmalloc(scal, sizeof(double) * 64));
-  C.part = (double*)part.p;
-  C.scal = (double*)scal.p;
-  D2_CUDA(cudaMallocHost(&C.hscal, sizeof(double) * 64));
-  struct PinnedFree {
-    double* p;
-    ~PinnedFree() { cudaFreeHost(p); }
-  } pf{C.hscal};
-  if (o.precision != DMRG2D_FP64) {
-    D2_TRY(dmalloc(lo, (o.precision == DMRG2D_BF16 ? 2 : 4) * (size_t)C.n));
-    D2_TRY(dmalloc(y32, sizeof(float) * (size_t)C.n));
-    C.lo = lo.p;
-    C.y32 = (float*)y32.p;
-  }
+  DevBuf buf;
+  const bool low = o.precision != DMRG2D_FP64;
+  D2_TRY(carve(buf, {{&C.part, sizeof(double) * (size_t)RED_BLOCKS * 520},
+                     {&C.scal, sizeof(double) * 64},
+                     {&C.lo, low ? (o.precision == DMRG2D_BF16 ? 2 : 4) * (size_t)C.n : 0},
+                     {&C.y32, low ? sizeof(float) * (size_t)C.n : 0}}));
+  PinnedSlot pinned;
+  D2_TRY(pinned.take(C.s));
+  C.hscal = pinned.p;
   int st;
   double energy = 0.0;
   D2_TRY(sec_zero_padding(ops, x_inout, C.s));  // restricted layouts: padding rows stay zero
@@ -2060,22 +2247,15 @@ extern "C" int dmrg2d_davidson_ground(const dmrg2d_ops* ops, const dmrg2d_davids
   C.s = (cudaStream_t)stream;
   C.n = ops->n_vec;
   C.st = &local;
-  DevBuf part, scal, lo, y32;
-  D2_TRY(dmalloc(part, sizeof(double) * (size_t)RED_BLOCKS * 520));
-  D2_TRY(dmalloc(scal, sizeof(double) * 64));
-  C.part = (double*)part.p;
-  C.scal = (double*)scal.p;
-  D2_CUDA(cudaMallocHost(&C.hscal, sizeof(double) * 64));
-  struct PinnedFree {
-    double* p;
-    ~PinnedFree() { cudaFreeHost(p); }
-  } pf{C.hscal};
-  if (o.precision != DMRG2D_FP64) {
-    D2_TRY(dmalloc(lo, (o.precision == DMRG2D_BF16 ? 2 : 4) * (size_t)C.n));
-    D2_TRY(dmalloc(y32, sizeof(float) * (size_t)C.n));
-    C.lo = lo.p;
-    C.y32 = (float*)y32.p;
-  }
+  DevBuf buf;
+  const bool low = o.precision != DMRG2D_FP64;
+  D2_TRY(carve(buf, {{&C.part, sizeof(double) * (size_t)RED_BLOCKS * 520},
+                     {&C.scal, sizeof(double) * 64},
+                     {&C.lo, low ? (o.precision == DMRG2D_BF16 ? 2 : 4) * (size_t)C.n : 0},
+                     {&C.y32, low ? sizeof(float) * (size_t)C.n : 0}}));
+  PinnedSlot pinned;
+  D2_TRY(pinned.take(C.s));
+  C.hscal = pinned.p;
   D2_TRY(sec_zero_padding(ops, x_inout, C.s));
   double energy = 0.0, resid = 0.0;
   int iters = 0;
