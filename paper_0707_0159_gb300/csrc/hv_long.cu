@@ -10,9 +10,9 @@
 // padded but the last 64 long indices.
 // Measured against one 64 x 64 piece per (row segment x column segment), whose padding was
 // the time (3-leg Hubbard superblock of 25 sectors, 4-leg Heisenberg of 7; moves included):
-//   Hubbard m = 256     FP64 115.6 -> 4.42 ms (1.01 TFLOP/s of 1.25), FP32 7.51 -> 0.98 ms
-//   Heisenberg m = 256  FP64 7.85 -> 4.13 ms,                         FP32 0.55 -> 0.51 ms
-//   Heisenberg m = 1024 FP64 275 -> 218 ms (1.23 TFLOP/s),            FP32 17.8 -> 15.9 ms
+//   Hubbard m = 256     FP64 115.6 -> 4.42 ms (1.01 TFLOP/s of 1.25), FP32 7.51 -> 0.51 ms
+//   Heisenberg m = 256  FP64 7.85 -> 4.13 ms,                         FP32 0.55 -> 0.20 ms
+//   Heisenberg m = 1024 FP64 275 -> 218 ms (1.23 TFLOP/s),            FP32 17.8 -> 7.0 ms
 #include <algorithm>
 
 #include "longplan.h"
@@ -197,15 +197,165 @@ hv_long_kernel(const T* __restrict__ v, T* __restrict__ y, const T* __restrict__
   }
 }
 
-template <typename T>
-int launch(const LongPlan* L, const T* v, T* y, const T* const* op, cudaStream_t s) {
-  const int n0 = (int)L->items[0].size(), n1 = (int)L->items[1].size();
-  if (n0)
-    hv_long_kernel<T, 0><<<n0, LT, 0, s>>>(v, y, op[0], L->d_items[0], L->d_segs[0], L->d_ks[0]);
-  if (n1)
-    hv_long_kernel<T, 1><<<n1, LT, 0, s>>>(v, y, op[1], L->d_items[1], L->d_segs[1], L->d_ks[1]);
-  D2_CUDA(cudaGetLastError());
-  return DMRG2D_OK;
+// FP32: the same passes in tiles of SEG segment indices by 2048 / SEG * 4 long ones, 8 long x
+// 4 segment outputs per thread, K chunks of 16 through registers.  Bound by the FP32 pipe
+// (SEG = 64: six wavefronts of shared memory per 32 FFMA of a warp) and, with narrow segments
+// (SEG = 16: nine), by shared memory.  Threads of one segment group fill whole or half warps,
+// so groups beyond a segment's end cost nothing.  Against the FP64 kernel's shape run in FP32
+// (16 outputs per thread in 8 x 2): Hubbard sectors m = 512 6.6 -> 2.0 ms, Heisenberg m = 1024
+// 15.9 -> 7.0 ms (38 TFLOP/s); dense 3-leg Hubbard m = 128, against 64 x 64 pieces, 12.4 ->
+// 5.8 ms (42 TFLOP/s).
+template <int PASS, int SEG>
+__device__ __forceinline__ void long_item32(const float* __restrict__ v, float* __restrict__ y,
+                                            const float* __restrict__ op, const LItem& it,
+                                            const LSeg& sg, const LK* __restrict__ ks,
+                                            float* __restrict__ Os, float* __restrict__ Vs, bool vec) {
+  constexpr int BK = 16, TL = 8192 / SEG, TX = TL / 8;  // long indices, threads along them
+  constexpr int NV = BK * TL / LT, NO = BK * SEG / LT;
+  constexpr int VS = TL + 4, OS = SEG + 4;
+  const int tid = threadIdx.x, tx = tid % TX, ty = tid / TX;
+  const int nx = min(TL, sg.nlong - it.x0);
+  const bool mine = 4 * ty < it.cnt && 4 * tx < nx;  // the second four long ones: + TL / 2
+  const long long ld = sg.ld;
+  float acc[8][4];
+#pragma unroll
+  for (int a = 0; a < 8; ++a)
+#pragma unroll
+    for (int b = 0; b < 4; ++b) acc[a][b] = 0.f;
+  float rv[NV], ro[NO];
+  const int kx = tid % BK, kr = tid / BK;
+  auto fetch = [&](const LK& k, int k0) {
+    const int kk = min(BK, k.kdim - k0);
+    const float* po = op + k.op + (long long)(it.s0 + kr) * k.kdim + k0 + kx;
+#pragma unroll
+    for (int r = 0; r < NO; ++r, po += (long long)(LT / BK) * k.kdim)
+      ro[r] = (kr + r * (LT / BK) < it.cnt && kx < kk) ? *po : 0.f;
+    if (PASS == 0) {  // V(x, k): rows are contiguous
+      if constexpr (TL >= LT) {
+#pragma unroll
+        for (int r = 0; r < NV; ++r) {
+          const int x = tid + (r % (TL / LT)) * LT, q = r / (TL / LT);
+          rv[r] = (x < nx && q < kk) ? v[sg.base + it.x0 + x + ld * (k.v_off + k0 + q)] : 0.f;
+        }
+      } else {
+        const float* p = v + sg.base + it.x0 + tid % TL + ld * (k.v_off + k0 + tid / TL);
+#pragma unroll
+        for (int r = 0; r < NV; ++r, p += ld * (LT / TL))
+          rv[r] = (tid % TL < nx && tid / TL + r * (LT / TL) < kk) ? *p : 0.f;
+      }
+    } else {  // V(k, x): the k of one column are contiguous
+      const float* p = v + sg.base + k.v_off + k0 + kx + ld * (it.x0 + kr);
+#pragma unroll
+      for (int r = 0; r < NV; ++r, p += ld * (LT / BK))
+        rv[r] = (kr + r * (LT / BK) < nx && kx < kk) ? *p : 0.f;
+    }
+  };
+  auto put = [&]() {
+#pragma unroll
+    for (int r = 0; r < NO; ++r) Os[kx * OS + kr + r * (LT / BK)] = ro[r];
+#pragma unroll
+    for (int r = 0; r < NV; ++r) {
+      if (PASS == 1)
+        Vs[kx * VS + kr + r * (LT / BK)] = rv[r];
+      else if constexpr (TL >= LT)
+        Vs[(r / (TL / LT)) * VS + tid + (r % (TL / LT)) * LT] = rv[r];
+      else
+        Vs[(tid / TL + r * (LT / TL)) * VS + tid % TL] = rv[r];
+    }
+  };
+  int e = sg.kb, k0 = 0;
+  LK k = e < sg.ke ? ks[e] : LK{0, 0, 0};
+  if (e < sg.ke) fetch(k, 0);
+  while (e < sg.ke) {
+    __syncthreads();
+    put();
+    __syncthreads();
+    k0 += BK;
+    if (k0 >= k.kdim) {
+      k0 = 0;
+      if (++e < sg.ke) k = ks[e];
+    }
+    if (e < sg.ke) fetch(k, k0);
+    if (mine) {
+#pragma unroll
+      for (int q = 0; q < BK; ++q) {
+        const float4 o = *(const float4*)(Os + q * OS + 4 * ty);
+        const float4 a0 = *(const float4*)(Vs + q * VS + 4 * tx);
+        const float4 a1 = *(const float4*)(Vs + q * VS + TL / 2 + 4 * tx);
+        const float av[8] = {a0.x, a0.y, a0.z, a0.w, a1.x, a1.y, a1.z, a1.w};
+        const float ov[4] = {o.x, o.y, o.z, o.w};
+#pragma unroll
+        for (int a = 0; a < 8; ++a)
+#pragma unroll
+          for (int b = 0; b < 4; ++b) acc[a][b] = fmaf(av[a], ov[b], acc[a][b]);
+      }
+    }
+  }
+  const int j0 = sg.off + it.s0 + 4 * ty, nj = min(4, it.cnt - 4 * ty);
+  if (mine) {
+    if (PASS == 0) {
+#pragma unroll
+      for (int b = 0; b < 4; ++b)
+#pragma unroll
+        for (int g = 0; g < 2; ++g) {
+          const int x = 4 * tx + g * (TL / 2);
+          float* Y = y + sg.base + it.x0 + x + ld * (j0 + b);
+          if (b < nj && vec && x + 3 < nx) {
+            *(float4*)Y = make_float4(acc[4 * g][b], acc[4 * g + 1][b], acc[4 * g + 2][b],
+                                      acc[4 * g + 3][b]);
+          } else if (b < nj) {
+#pragma unroll
+            for (int a = 0; a < 4; ++a)
+              if (x + a < nx) Y[a] = acc[4 * g + a][b];
+          }
+        }
+    } else {
+#pragma unroll
+      for (int a = 0; a < 8; ++a) {
+        const int x = 4 * tx + (a / 4) * (TL / 2) + a % 4;
+        if (x >= nx) continue;
+        float* Y = y + sg.base + j0 + ld * (it.x0 + x);
+        if (vec && nj == 4) {
+          float4 o = *(const float4*)Y;
+          o.x += acc[a][0];
+          o.y += acc[a][1];
+          o.z += acc[a][2];
+          o.w += acc[a][3];
+          *(float4*)Y = o;
+        } else {
+#pragma unroll
+          for (int b = 0; b < 4; ++b)
+            if (b < nj) Y[b] += acc[a][b];
+        }
+      }
+    }
+  }
+  if (PASS == 1 && it.s0 + it.cnt == sg.dim)  // the segment's padding rows
+    for (int x = tid; x < nx; x += LT)
+      for (int j = sg.dim; j < sg.dim_pad; ++j) y[sg.base + sg.off + j + ld * (it.x0 + x)] = 0.f;
+}
+
+// long indices of an FP32 item of cnt segment indices
+int long_of32(int cnt) { return cnt <= 16 ? 512 : cnt <= 32 ? 256 : 128; }
+
+template <int PASS>
+__global__ void __launch_bounds__(LT, 2)
+hv_long32_kernel(const float* __restrict__ v, float* __restrict__ y, const float* __restrict__ op,
+                 const LItem* __restrict__ items, const LSeg* __restrict__ segs,
+                 const LK* __restrict__ ks) {
+  __shared__ __align__(16) float Os[16 * (LP_ROWS + 4)];
+  __shared__ __align__(16) float Vs[16 * (512 + 4)];
+  const LItem it = items[blockIdx.x];
+  const LSeg sg = segs[it.seg];
+  // 16-byte accesses to y: first element and leading dimension multiples of four
+  const bool vec = ((((uintptr_t)y >> 2) | (uintptr_t)sg.base | (uintptr_t)sg.ld |
+                     (uintptr_t)(PASS == 0 ? it.x0 : sg.off + it.s0)) & 3) == 0;
+  if (it.cnt <= 16)
+    long_item32<PASS, 16>(v, y, op, it, sg, ks, Os, Vs, vec);
+  else if (it.cnt <= 32)
+    long_item32<PASS, 32>(v, y, op, it, sg, ks, Os, Vs, vec);
+  else
+    long_item32<PASS, 64>(v, y, op, it, sg, ks, Os, Vs, vec);
 }
 
 // Four rows of a column, n of them inside the matrix (VEC: all four, aligned).
@@ -346,6 +496,7 @@ int lp_finalise(dmrg2d_ops* ops, LongPlan* L, cudaStream_t s) {
       while ((kt >> sg.head) > 4096) ++sg.head;
     }
     L->items[ps] = cut(L, ps, LP_ROWS, 1, [](int cnt) { return 64 * (8 / row_groups(cnt)); });
+    L->items32[ps] = cut(L, ps, LP_ROWS, 4, long_of32);
     // narrower items where 64 indices by 128 would leave SMs without one
     for (int cap = LP_ROWS; cap >= 16; cap /= 2) {
       L->fitems[ps] = cut(L, ps, cap, 8, [](int) { return FX_LONG; });
@@ -356,6 +507,7 @@ int lp_finalise(dmrg2d_ops* ops, LongPlan* L, cudaStream_t s) {
     D2_TRY(up(L, L->ks[ps], &L->d_ks[ps], nb, s));
     D2_TRY(up(L, L->units[ps], &L->d_units[ps], nb, s));
     D2_TRY(up(L, L->items[ps], &L->d_items[ps], nb, s));
+    D2_TRY(up(L, L->items32[ps], &L->d_items32[ps], nb, s));
     D2_TRY(up(L, L->fitems[ps], &L->d_fitems[ps], nb, s));
     D2_TRY(up(L, std::vector<int>((size_t)e0, 0), &L->d_opE[ps], nb, s));
   }
@@ -383,10 +535,26 @@ int lp_read_error(const LongPlan* L, int* code) {
 }
 
 int lp_launch_f64(const LongPlan* L, const double* v, double* y, cudaStream_t s) {
-  return launch<double>(L, v, y, L->op64, s);
+  const int n0 = (int)L->items[0].size(), n1 = (int)L->items[1].size();
+  if (n0)
+    hv_long_kernel<double, 0><<<n0, LT, 0, s>>>(v, y, L->op64[0], L->d_items[0], L->d_segs[0],
+                                                L->d_ks[0]);
+  if (n1)
+    hv_long_kernel<double, 1><<<n1, LT, 0, s>>>(v, y, L->op64[1], L->d_items[1], L->d_segs[1],
+                                                L->d_ks[1]);
+  D2_CUDA(cudaGetLastError());
+  return DMRG2D_OK;
 }
 int lp_launch_f32(const LongPlan* L, const float* v, float* y, cudaStream_t s) {
-  return launch<float>(L, v, y, L->op32, s);
+  const int n0 = (int)L->items32[0].size(), n1 = (int)L->items32[1].size();
+  if (n0)
+    hv_long32_kernel<0><<<n0, LT, 0, s>>>(v, y, L->op32[0], L->d_items32[0], L->d_segs[0],
+                                          L->d_ks[0]);
+  if (n1)
+    hv_long32_kernel<1><<<n1, LT, 0, s>>>(v, y, L->op32[1], L->d_items32[1], L->d_segs[1],
+                                          L->d_ks[1]);
+  D2_CUDA(cudaGetLastError());
+  return DMRG2D_OK;
 }
 int lp_moves_f64(const LongPlan* L, const double* v, double* y, cudaStream_t s) {
   return moves(L, v, y, s);

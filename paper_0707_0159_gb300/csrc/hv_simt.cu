@@ -281,8 +281,13 @@ int launch(const dmrg2d_ops* ops, const T* v, T* y, const T* HL, const T* HR, co
     two_pass = (int)ops->lp->items[0].size() >= 2 * sms &&
                1.1 * (double)ops->n_vec / sms < 0.98 * best;
   } else {
-    // the largest piece (64, 32 or 16 square) whose grid still gives every SM a CTA
+    // the largest piece (64, 32 or 16 square) whose grid still gives every SM a CTA; the
+    // two-pass kernel's larger register tiles once they fill nearly half of the SMs (2-leg
+    // 100 x 128, 32 items: 66 us in pieces, 67 two-pass; 2-leg Hubbard 40 x 40, 80 items: 80
+    // and 48 us; 3-leg Heisenberg 250 x 131: 641 and 295 us; 3-leg Hubbard 128 x 128: 12.4
+    // and 5.8 ms)
     tb = ctas(64) >= sms ? 64 : (ctas(32) >= sms ? 32 : 16);
+    two_pass = 5 * (int)ops->lp->items32[0].size() >= 2 * sms;
   }
   const int64_t gx = (int64_t)((ops->m1 + tb - 1) / tb) * ops->d;
   const int64_t gy = (int64_t)((ops->m4 + tb - 1) / tb) * ops->d;
@@ -292,11 +297,15 @@ int launch(const dmrg2d_ops* ops, const T* v, T* y, const T* HL, const T* HR, co
   dim3 grid((unsigned)gx, (unsigned)gy);
   auto ev = prof_slot(ops);
   if (ev.first) D2_CUDA(cudaEventRecord(ev.first, s));
-  if constexpr (sizeof(T) == 8) {
-    if (two_pass) {
+  if (two_pass) {
+    if constexpr (sizeof(T) == 8) {
       D2_TRY(lp_launch_f64(ops->lp, v, y, s));
       if (ev.second) D2_CUDA(cudaEventRecord(ev.second, s));
       return lp_moves_f64(ops->lp, v, y, s);
+    } else {
+      D2_TRY(lp_launch_f32(ops->lp, v, y, s));
+      if (ev.second) D2_CUDA(cudaEventRecord(ev.second, s));
+      return lp_moves_f32(ops->lp, v, y, s);
     }
   }
   if (tb == 64)

@@ -60,11 +60,11 @@ struct LongPlan {
   const float *op32[2] = {nullptr, nullptr};
   // derived (lp_finalise)
   std::vector<LUnit> units[2];
-  std::vector<LItem> items[2], fitems[2];
+  std::vector<LItem> items[2], items32[2], fitems[2];  // FP64, FP32, FP64X
   LSeg* d_segs[2] = {nullptr, nullptr};
   LK* d_ks[2] = {nullptr, nullptr};
   LUnit* d_units[2] = {nullptr, nullptr};
-  LItem *d_items[2] = {nullptr, nullptr}, *d_fitems[2] = {nullptr, nullptr};
+  LItem *d_items[2] = {nullptr, nullptr}, *d_items32[2] = {nullptr, nullptr}, *d_fitems[2] = {nullptr, nullptr};
   int* d_opE[2] = {nullptr, nullptr};  // largest exponent field of every operator row
   MoveRec* d_mrec = nullptr;
   MoveItem* d_mitems = nullptr;

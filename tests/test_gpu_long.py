@@ -83,6 +83,23 @@ def test_fp64x_dense_sizes(legs, m1, m4):
     assert rel(got, sb.apply(v)) <= 1e-12
 
 
+@pytest.mark.parametrize("prec,tol", [(dmrg2d.FP64, 1e-12), (dmrg2d.FP32, 1e-5)])
+@pytest.mark.parametrize("kind,legs,m1,m4", [
+    ("heisenberg", 2, 7, 9), ("heisenberg", 2, 64, 64), ("heisenberg", 3, 70, 65),
+    ("heisenberg", 3, 131, 100), ("hubbard", 2, 10, 10), ("hubbard", 2, 41, 38),
+    ("heisenberg", 5, 33, 3)])
+def test_dense_kernel_choice(kind, legs, m1, m4, prec, tol):
+    """Every piece size and the two-pass kernel of the dense CUDA-core H.v."""
+    make = synth.heisenberg_block if kind == "heisenberg" else synth.hubbard_block
+    mdl, left, right = synth.model(kind, legs), make(m1, legs, 3), make(m4, legs, 4)
+    sb = Superblock(mdl, left, right)
+    v = synth.start_vector(sb.n_vec, 9)
+    x = torch.from_numpy(v).to("cuda", torch.float64 if prec == dmrg2d.FP64 else torch.float32)
+    y = torch.full_like(x, 7.0)
+    dmrg2d.apply_H(dmrg2d.build_ops(mdl, left, right), x, y, prec)
+    assert rel(y.double().cpu().numpy(), sb.apply(v)) <= tol
+
+
 @pytest.fixture(scope="module")
 def hubbard2():
     mdl = synth.model("hubbard", 2, t=1.0, U=6.0)
