@@ -369,6 +369,7 @@ hv_tc_grouped_kernel(const __grid_constant__ GMaps maps, const GParams p) {
 struct SItem {
   int q, seg, n0, m0;  // matrix; segment (row segment in pass 1, column segment in pass 2);
                        // offset of the N range in the segment; first of the 128 M indices
+  int kb, ke, sdim, pad;  // the segment's operator blocks and extent
 };
 
 struct SParams {
@@ -432,63 +433,71 @@ hv_tc_seg_kernel(const __grid_constant__ GMaps maps, const SParams p) {
   const uint32_t tmem_base = *tmem_slot;
   const int BK = p.BK;
 
-  if (warp == 0 && lane == 0) {
+  // The operator-block entries of a piece are read by the whole warp, one per lane, and those
+  // of the next piece while this one runs: read one after another by the issuing thread, each
+  // was a global-memory latency in front of the one or two stages of its block (3-leg Hubbard
+  // sectors, m = 1024, TF32 H·v: 3.87 -> 3.44 ms; the two passes now read 9 and 11 GB at 8 TB/s
+  // from L2, a third of it padding of K = 41 to 64).
+  // {a_pool, b_row, kdim, neg} in pass 1, {a_col, b_pool, kdim, neg} in pass 2
+  const int4* const ents = PASS == 0 ? (const int4*)p.k1 : (const int4*)p.k2;
+  const SItem none = {0, 0, 0, 0, 0, 0, 0, 0};
+  if (warp == 0) {
     // ------------------------------- TMA producer -------------------------------
     int stage = 0;
     uint32_t phase = 0;
-    for (int ti = blockIdx.x; ti < p.nitems && !*abort; ti += gridDim.x) {
-      const SItem it = p.items[ti];
-      const int e0 = PASS == 0 ? p.rows[it.seg].k1b : p.cols[it.seg].k2b;
-      const int e1 = PASS == 0 ? p.rows[it.seg].k1e : p.cols[it.seg].k2e;
+    bool ok = true;
+    int ti = blockIdx.x;
+    SItem it = ti < p.nitems ? p.items[ti] : none;
+    int4 ent = it.kb + lane < it.ke ? ents[it.kb + lane] : make_int4(0, 0, 0, 0);
+    for (; ti < p.nitems && ok; ti += gridDim.x) {
+      const SItem nx = ti + (int)gridDim.x < p.nitems ? p.items[ti + gridDim.x] : none;
+      int4 ent_nx = make_int4(0, 0, 0, 0);
       // the operator rows this piece needs, in 32-row boxes (N rounded up to 16 <= 32 nb)
-      const int sdim = PASS == 0 ? p.rows[it.seg].dim : p.cols[it.seg].dim;
-      const int nb = (min(NMAX, sdim - it.n0) + 31) / 32;
+      const int nb = (min(NMAX, it.sdim - it.n0) + 31) / 32;
       const uint32_t tx = p.a_bytes + (uint32_t)nb * p.b_box_bytes;
-      for (int e = e0; e < e1; ++e) {
-        int kdim, pool, voff;
-        if (PASS == 0) {
-          const GK1 k = p.k1[e];
-          kdim = k.kdim;
-          pool = k.a_pool;
-          voff = k.b_row;
-        } else {
-          const GK2 k = p.k2[e];
-          kdim = k.kdim;
-          pool = k.b_pool;
-          voff = k.a_col;
-        }
+      // lane b copies box b: the V tile's (pass 1: one, rows voff .. (K) by columns m0 .. (M);
+      // pass 2: 32-row boxes of rows m0 .. (M, MN-major) by columns voff .. (K)), then the
+      // operator rows', 32 at a time (the 128B swizzle is a function of the shared-memory
+      // address, so the boxes line up as one tile)
+      const int na = PASS == 0 ? 1 : p.a2_boxes, bi = lane - na;
+      for (int e = it.kb; e < it.ke && ok; ++e) {
+        const int le = (e - it.kb) & 31;
+        if (le == 0 && e > it.kb)
+          ent = e + lane < it.ke ? ents[e + lane] : make_int4(0, 0, 0, 0);
+        if (e == it.kb && nx.kb + lane < nx.ke) ent_nx = ents[nx.kb + lane];
+        const int f0 = __shfl_sync(0xffffffffu, ent.x, le), f1 = __shfl_sync(0xffffffffu, ent.y, le);
+        const int kdim = __shfl_sync(0xffffffffu, ent.z, le);
+        const int pool = PASS == 0 ? f0 : f1, voff = PASS == 0 ? f1 : f0;
         const int nk = (kdim + BK - 1) / BK;
         for (int kc = 0; kc < nk; ++kc) {
-          if (!mbar_wait(empty(stage), phase ^ 1u, abort)) {
-            raise_abort(abort, p.err, 21);
-            goto producer_done;
+          ok = __all_sync(0xffffffffu, mbar_wait(empty(stage), phase ^ 1u, abort));
+          if (!ok) {
+            if (lane == 0) raise_abort(abort, p.err, 21);
+            break;
           }
           const uint32_t a_s = smem_u32(smem + stage * G_STAGE);
           const uint32_t b_s = a_s + G_STAGE_A;
-          mbar_expect_tx(full(stage), tx);
-          if (PASS == 0) {
-            // A: V_q rows voff + kc BK .. (K), columns m0 .. m0 + 127 (M)
-            tma_load_2d(a_s, &maps.vk[it.q], full(stage), voff + kc * BK, it.m0);
-          } else {
-            // A: V_q rows m0 .. m0 + 127 (M, MN-major), columns voff + kc BK .. (K)
-            for (int b = 0; b < p.a2_boxes; ++b)
-              tma_load_2d(a_s + b * p.a2_lbo, &maps.vm[it.q], full(stage),
-                          it.m0 + b * p.a2_box_rows, voff + kc * BK);
+          if (lane == 0) mbar_expect_tx(full(stage), tx);
+          __syncwarp();
+          if (bi < 0) {
+            if (PASS == 0)
+              tma_load_2d(a_s, &maps.vk[it.q], full(stage), voff + kc * BK, it.m0);
+            else
+              tma_load_2d(a_s + lane * p.a2_lbo, &maps.vm[it.q], full(stage),
+                          it.m0 + lane * p.a2_box_rows, voff + kc * BK);
+          } else if (bi < nb) {
+            tma_load_2d(b_s + bi * 32 * 128, PASS == 0 ? &maps.L : &maps.R, full(stage), kc * BK,
+                        pool + it.n0 + 32 * bi);
           }
-          // B: operator rows pool + n0 .., 32 at a time (the 128B swizzle is a function of
-          // the shared-memory address, so the boxes line up as one tile)
-          for (int b = 0; b < nb; ++b)
-            tma_load_2d(b_s + b * 32 * 128, PASS == 0 ? &maps.L : &maps.R, full(stage), kc * BK,
-                        pool + it.n0 + 32 * b);
-          if (++stage == G_STAGES) {
-            stage = 0;
-            phase ^= 1u;
-          }
+          stage = stage + 1 == G_STAGES ? 0 : stage + 1;
+          phase ^= stage == 0 ? 1u : 0u;
         }
       }
+      if (it.kb == it.ke && nx.kb + lane < nx.ke) ent_nx = ents[nx.kb + lane];
+      it = nx;
+      ent = ent_nx;
     }
-  producer_done:;
-  } else if (warp == 1 && lane == 0) {
+  } else if (warp == 1) {
     // ------------------------------- MMA issuer ---------------------------------
     int stage = 0;
     uint32_t phase = 0;
@@ -498,31 +507,37 @@ hv_tc_seg_kernel(const __grid_constant__ GMaps maps, const SParams p) {
     const uint32_t a_step = PASS == 0 ? 32u : p.a2_kstep;
     const uint64_t b_hi = sdesc(0, 16, 1024);
     const int ksteps = BK / p.KSTEP;  // 4
-    for (int ti = blockIdx.x; ti < p.nitems && !*abort; ti += gridDim.x) {
-      const SItem it = p.items[ti];
-      const int sdim = PASS == 0 ? p.rows[it.seg].dim : p.cols[it.seg].dim;
-      const int nvalid = min(NMAX, sdim - it.n0);
-      const int nidx = (nvalid + 15) / 16 - 1;
-      const int e0 = PASS == 0 ? p.rows[it.seg].k1b : p.cols[it.seg].k2b;
-      const int e1 = PASS == 0 ? p.rows[it.seg].k1e : p.cols[it.seg].k2e;
-      if (!mbar_wait(tempty(acc), aphase ^ 1u, abort)) {
-        raise_abort(abort, p.err, 22);
+    const uint32_t el = lane == 0;
+    bool ok = true;
+    int ti = blockIdx.x;
+    SItem it = ti < p.nitems ? p.items[ti] : none;
+    int4 ent = it.kb + lane < it.ke ? ents[it.kb + lane] : make_int4(0, 0, 0, 0);
+    for (; ti < p.nitems && ok; ti += gridDim.x) {
+      const SItem nx = ti + (int)gridDim.x < p.nitems ? p.items[ti + gridDim.x] : none;
+      int4 ent_nx = make_int4(0, 0, 0, 0);
+      const int nidx = (min(NMAX, it.sdim - it.n0) + 15) / 16 - 1;
+      ok = __all_sync(0xffffffffu, mbar_wait(tempty(acc), aphase ^ 1u, abort));
+      if (!ok) {
+        if (lane == 0) raise_abort(abort, p.err, 22);
         break;
       }
       tc_fence_after();
       const uint32_t dt = tmem_base + acc * G_ACC_COLS;
       uint32_t accum = 0;
-      bool ok = true;
-      for (int e = e0; e < e1 && ok; ++e) {
-        const int kdim = PASS == 0 ? p.k1[e].kdim : p.k2[e].kdim;
-        const int neg = PASS == 0 ? p.k1[e].neg : p.k2[e].neg;
+      for (int e = it.kb; e < it.ke && ok; ++e) {
+        const int le = (e - it.kb) & 31;
+        if (le == 0 && e > it.kb)
+          ent = e + lane < it.ke ? ents[e + lane] : make_int4(0, 0, 0, 0);
+        if (e == it.kb && nx.kb + lane < nx.ke) ent_nx = ents[nx.kb + lane];
+        const int kdim = __shfl_sync(0xffffffffu, ent.z, le);
+        const int neg = __shfl_sync(0xffffffffu, ent.w, le);
         const uint32_t id = p.idesc[nidx][neg];
         const int nk = (kdim + BK - 1) / BK;
         const int last = (kdim - (nk - 1) * BK + p.KSTEP - 1) / p.KSTEP;  // steps in the last stage
         for (int kc = 0; kc < nk; ++kc) {
-          if (!mbar_wait(full(stage), phase, abort)) {
-            raise_abort(abort, p.err, 23);
-            ok = false;
+          ok = __all_sync(0xffffffffu, mbar_wait(full(stage), phase, abort));
+          if (!ok) {
+            if (lane == 0) raise_abort(abort, p.err, 23);
             break;
           }
           const uint32_t a_s = smem_u32(smem + stage * G_STAGE);
@@ -531,21 +546,25 @@ hv_tc_seg_kernel(const __grid_constant__ GMaps maps, const SParams p) {
 #pragma unroll
           for (int k = 0; k < 4; ++k) {
             umma_if_t<BF16>(dt, a_hi | sdesc_addr(a_s + k * a_step), b_hi | sdesc_addr(b_s + k * 32),
-                            id, accum, (uint32_t)(k < nks));
+                            id, accum, (uint32_t)(k < nks) & el);
             accum = 1;  // step 0 is always issued
           }
-          umma_commit(empty(stage));
+          if (el) umma_commit(empty(stage));
           stage = stage + 1 == G_STAGES ? 0 : stage + 1;
           phase ^= stage == 0 ? 1u : 0u;
         }
       }
       if (!ok) break;
-      umma_commit(tfull(acc));
+      if (el) umma_commit(tfull(acc));
       if (++acc == 2) {
         acc = 0;
         aphase ^= 1u;
       }
+      if (it.kb == it.ke && nx.kb + lane < nx.ke) ent_nx = ents[nx.kb + lane];
+      it = nx;
+      ent = ent_nx;
     }
+    __syncwarp();
   } else if (warp >= 2) {
     // ------------------------------- epilogue -----------------------------------
     // TMEM lane = M index (a column of V_q in pass 1, a row in pass 2), TMEM column = N
@@ -616,11 +635,15 @@ hv_tc_seg_kernel(const __grid_constant__ GMaps maps, const SParams p) {
           uint32_t v[32];
           tmem_ld32(tmem_base + acc * G_ACC_COLS + ((uint32_t)(32 * q4) << 16) + ch * 32, v);
           if (row_ok) {
+            // all reads of Y before the first write: interleaved, each pair waited for the one
+            // before it (pass 2 of the 3-leg Hubbard sectors, m = 1024: 3.27 -> 1.7 ms)
+            float o[32];
 #pragma unroll
-            for (int j = 0; j < 32; ++j) {
-              const int n = ch * 32 + j;
-              if (n < nval) yrow[ld * n] += __uint_as_float(v[j]);
-            }
+            for (int j = 0; j < 32; ++j)
+              o[j] = ch * 32 + j < nval ? yrow[ld * (ch * 32 + j)] : 0.f;
+#pragma unroll
+            for (int j = 0; j < 32; ++j)
+              if (ch * 32 + j < nval) yrow[ld * (ch * 32 + j)] = o[j] + __uint_as_float(v[j]);
           }
         }
       }
@@ -753,6 +776,34 @@ std::pair<int, int> BlockPool::add(const double* src, int rows, int cols, int64_
   return {(int)ent.size() - 1, 0};
 }
 
+void gp_stage_bytes(const GroupPlan* g, int bk, double* grouped, double* segment) {
+  auto up = [](int a, int b) { return (double)((a + b - 1) / b); };
+  struct Sum {
+    double pieces = 0, stages = 0;  // pieces; pieces times stages of their block lists
+  };
+  std::vector<Sum> r(g->nQ), c(g->nQ);
+  *segment = 0;
+  for (const GRow& s : g->rows) {
+    double k = 0;
+    for (int e = s.k1b; e < s.k1e; ++e) k += up(g->k1[e].kdim, bk);
+    r[s.q].pieces += up(s.dim, G_BM);
+    r[s.q].stages += up(s.dim, G_BM) * k;
+    *segment += up(g->qcols[s.q], 128) * up(s.dim, 128) * k *
+                (G_STAGE_A + 4096 * up(std::min(s.dim, 128), 32));
+  }
+  for (const GCol& s : g->cols) {
+    double k = 0;
+    for (int e = s.k2b; e < s.k2e; ++e) k += up(g->k2[e].kdim, bk);
+    c[s.q].pieces += up(s.dim, 256);
+    c[s.q].stages += up(s.dim, 256) * k;
+    *segment += up(g->qld[s.q], 128) * up(s.dim, 256) * k *
+                (G_STAGE_A + 4096 * up(std::min(s.dim, 256), 32));
+  }
+  *grouped = 0;
+  for (int q = 0; q < g->nQ; ++q)
+    *grouped += (r[q].stages * c[q].pieces + r[q].pieces * c[q].stages) * G_STAGE;
+}
+
 int gp_num_configs() { return 2 * N_ORDERS; }
 const char* gp_config_name(int cfg) {
   return cfg >= 0 && cfg < 2 * N_ORDERS ? kNames[cfg] : "?";
@@ -863,12 +914,12 @@ int gp_finalise(dmrg2d_ops* ops, GroupPlan* g, cudaStream_t s) {
       for (int m0 = 0; m0 < g->qcols[q]; m0 += 128)
         for (size_t r = 0; r < g->rows.size(); ++r) {
           if (g->rows[r].q != q) continue;
-          for (int n0 = 0; n0 < g->rows[r].dim; n0 += 128) s1.push_back({q, (int)r, n0, m0});
+          for (int n0 = 0; n0 < g->rows[r].dim; n0 += 128) s1.push_back({q, (int)r, n0, m0, g->rows[r].k1b, g->rows[r].k1e, g->rows[r].dim, 0});
         }
       for (int m0 = 0; m0 < g->qld[q]; m0 += 128)
         for (size_t c = 0; c < g->cols.size(); ++c) {
           if (g->cols[c].q != q) continue;
-          for (int n0 = 0; n0 < g->cols[c].dim; n0 += 256) s2.push_back({q, (int)c, n0, m0});
+          for (int n0 = 0; n0 < g->cols[c].dim; n0 += 256) s2.push_back({q, (int)c, n0, m0, g->cols[c].k2b, g->cols[c].k2e, g->cols[c].dim, 0});
         }
     }
     st = gup(D, s1, &D->sitems[0], nb, s);

@@ -85,6 +85,9 @@ int gp_launch(const dmrg2d_ops* ops, const GroupPlan* g, const void* v, float* y
 // No scalar moves.  y must be 16-byte aligned.
 int gp_launch_seg(const dmrg2d_ops* ops, const GroupPlan* g, const void* v, float* y,
                   int precision, cudaStream_t s, bool lo_ops = false, bool accum = false);
+// bytes that the pipeline stages of the grouped kernel (128 x 256 pieces) and of the segment
+// kernels read per H·v (K per stage: 32 TF32 or 64 BF16)
+void gp_stage_bytes(const GroupPlan* g, int bk, double* grouped, double* segment);
 int gp_read_error(const GroupPlan* g, int* code);
 // pool tensor maps and per-block entries (CSR order of the build) for another kernel
 int gp_pool_views(const GroupPlan* g, int precision, int bn, const CUtensorMap** mL,
