@@ -419,7 +419,7 @@ static int long_prepare(dmrg2d_ops* ops, cudaStream_t s) {
   auto at = [&](int t) { return (long long)(t % d) * m1 + (long long)ld * (t / d) * m4; };
   for (int t = 0; t < d * d; ++t)
     if (ops->hCptr[t + 1] > ops->hCptr[t])
-      lp_add_moves(L, at(t), ld, m1, m1, m4, ops->hCptr[t], ops->hCptr[t + 1]);
+      lp_add_moves(L, 0, at(t), ld, m1, m1, m4, ops->hCptr[t], ops->hCptr[t + 1]);
   for (int e = 0; e < D.nC; ++e)
     L->mrec.push_back({at(ops->hCsrc[e]), ld, (float)ops->hCval[e], ops->hCval[e]});
   L->quads = m1 % 4 == 0;

@@ -105,6 +105,7 @@ struct dmrg2d_ops {
   // tensor-core kernel choice per precision: -1 the dense kernel, >= 0 a grouped-kernel
   // tile configuration (set by dmrg2d_autotune; defaults chosen at build time)
   int tc_cfg[4] = {-1, -1, -1, -1};
+  bool tc_chosen[4] = {false, false, false, false};  // set by the caller or the autotuner
   // kernel timing (dmrg2d_profile_start/stop); apply_H only records into it
   mutable std::vector<std::pair<cudaEvent_t, cudaEvent_t>> prof_ev;
   mutable size_t prof_used = 0;

@@ -389,6 +389,9 @@ __device__ __forceinline__ void load4(const Tin* p, int n, Tout (&o)[4]) {
 // move) left most lanes of a small sector idle: on the 4-leg Heisenberg sectors of m = 1024
 // the whole BF16 H·v went from 958 to 675 us, on the 3-leg Hubbard ones in TF32 from 5.92
 // to 5.33 ms (there the tile configuration with separate moves became the faster one).
+// The items run group by group (all blocks that exchange elements, a few MB): every source
+// comes from L2 after its first use.  In the order of the vector each of the 3-4 sources of
+// an element was a read from memory: 0.89 -> 0.69 ms on the 3-leg Hubbard sectors in TF32.
 constexpr int MV_THREADS = 128, MV_ITEMS = 1024;  // threads; fours of rows per block
 template <typename Tin, typename Tout, bool VEC>
 __global__ void __launch_bounds__(MV_THREADS)
@@ -468,11 +471,12 @@ int up(LongPlan* L, const std::vector<T>& h, T** d, int64_t* bytes, cudaStream_t
 
 }  // namespace
 
-void lp_add_moves(LongPlan* L, long long dst, int ld, int dim, int dim_pad, int ncols, int mb,
-                  int me) {
+void lp_add_moves(LongPlan* L, int group, long long dst, int ld, int dim, int dim_pad, int ncols,
+                  int mb, int me) {
   const int nquad = (dim_pad + 3) / 4, step = std::max(1, MV_ITEMS / nquad);
   for (int c = 0; c < ncols; c += step)
-    L->mitems.push_back({dst, ld, dim, nquad, c, std::min(step, ncols - c), mb, me});
+    L->mitems.push_back({dst, ld, dim, nquad, c, std::min(step, ncols - c), mb, me,
+                         ((long long)group << 32) + c});
 }
 
 int lp_finalise(dmrg2d_ops* ops, LongPlan* L, cudaStream_t s) {
@@ -511,6 +515,8 @@ int lp_finalise(dmrg2d_ops* ops, LongPlan* L, cudaStream_t s) {
     D2_TRY(up(L, L->fitems[ps], &L->d_fitems[ps], nb, s));
     D2_TRY(up(L, std::vector<int>((size_t)e0, 0), &L->d_opE[ps], nb, s));
   }
+  std::stable_sort(L->mitems.begin(), L->mitems.end(),
+                   [](const MoveItem& a, const MoveItem& b) { return a.group < b.group; });
   D2_TRY(up(L, L->mrec, &L->d_mrec, &ops->device_bytes, s));
   D2_TRY(up(L, L->mitems, &L->d_mitems, &ops->device_bytes, s));
   D2_TRY(up(L, std::vector<int>(1, 0), &L->err, &ops->device_bytes, s));

@@ -1235,6 +1235,7 @@ extern "C" int dmrg2d_set_tile_config(dmrg2d_ops* ops, int precision, int index)
   if (!tc_candidate_ok(ops, index))
     return set_error(DMRG2D_EUNSUPPORTED, "tile configuration %d not available here", index);
   ops->tc_cfg[precision] = idx_to_cfg(index);
+  ops->tc_chosen[precision] = true;
   return DMRG2D_OK;
 }
 
@@ -1309,6 +1310,7 @@ extern "C" int dmrg2d_autotune(dmrg2d_ops* ops, int precision, int* best, double
   if (derr) return set_error(DMRG2D_ETIMEOUT, "tensor-core kernel gave up waiting (site %d)", derr);
   if (chosen < 0) return set_error(DMRG2D_EUNSUPPORTED, "no tile configuration applies");
   ops->tc_cfg[precision] = idx_to_cfg(chosen);
+  ops->tc_chosen[precision] = true;
   if (best) *best = chosen;
   return DMRG2D_OK;
 }

@@ -48,6 +48,7 @@ struct MoveItem {   // columns c_in .. c_in + ncol of a destination block
   long long dst;    // its first element
   int ld, dim, nquad;  // leading dimension, rows, fours of rows (with padding)
   int c_in, ncol, mb, me;  // moves[mb..me)
+  long long group;  // blocks of one group share their sources
 };
 
 struct LongPlan {
@@ -73,9 +74,11 @@ struct LongPlan {
   std::vector<void*> allocs;
 };
 
-// Moves of one destination block: appends its items (columns in chunks).
-void lp_add_moves(LongPlan* L, long long dst, int ld, int dim, int dim_pad, int ncols, int mb,
-                  int me);
+// Moves of one destination block: appends its items (columns in chunks).  A move keeps the
+// block-1 and the block-4 sector, so all sources of a block lie in its `group` (one per pair
+// of sectors); lp_finalise orders the items by group and chunk.
+void lp_add_moves(LongPlan* L, int group, long long dst, int ld, int dim, int dim_pad, int ncols,
+                  int mb, int me);
 // Cuts the segments into items and uploads everything; op64 / op32 must be set.
 int lp_finalise(dmrg2d_ops* ops, LongPlan* L, cudaStream_t s);
 void lp_release(LongPlan* L);

@@ -112,6 +112,24 @@ int up(SecState* S, const std::vector<T>& h, T** d, int64_t* bytes, cudaStream_t
 
 }  // namespace
 
+// Grouped layout of a sector superblock: 128 x 256 pieces, longest first, with the scalar moves
+// in the epilogue (TF32) or in their own kernel (BF16, whose epilogue converts every source:
+// 4-leg Heisenberg, m = 1024, 1.49 against 0.63 ms; TF32 0.93 against 1.01 ms).
+static int grouped_cfg(int precision) {
+  return precision == DMRG2D_BF16 ? gp_num_configs() + 5 : 5;
+}
+// The configuration before any autotuning: the segment kernels where the grouped kernel's
+// stages would read more than 2.5 times their bytes (its pieces pad narrow sectors on both
+// sides) and the superblock is large enough for their two passes.  Grouped / segment bytes and
+// times, TF32: 4-leg Heisenberg m = 384 2.1 / 0.72 GB, 0.167 / 0.146 ms; m = 512 2.6 / 1.3 GB,
+// 0.204 / 0.223 ms; 2-leg m = 256 0.05 / 0.01 GB, 0.021 / 0.032 ms; 2-leg Hubbard m = 256 2.0 /
+// 0.12 GB, 0.184 / 0.049 ms; 3-leg Hubbard m = 1024 6.0 / 3.2 ms.
+static int default_cfg(const GroupPlan* g, int precision) {
+  double grouped, segment;
+  gp_stage_bytes(g, precision == DMRG2D_BF16 ? 64 : 32, &grouped, &segment);
+  return segment < 0.4 * grouped && grouped > 3e8 ? 2 * gp_num_configs() : grouped_cfg(precision);
+}
+
 int sec_build(dmrg2d_ops* ops, const dmrg2d_block* L, const dmrg2d_block* R, const int32_t* target,
               const std::vector<double>& HL, const std::vector<double>& HR, cudaStream_t s) {
   const int d = ops->d, m1 = ops->m1, m4 = ops->m4;
@@ -310,7 +328,7 @@ int sec_build(dmrg2d_ops* ops, const dmrg2d_block* L, const dmrg2d_block* R, con
       S->mdst.push_back(md);
       const RowSegD& rs = S->rseg[r];
       const ColSegD& cs = S->cseg[c];
-      lp_add_moves(lp, S->qbase[rs.q] + rs.off + (long long)S->qld[rs.q] * cs.off, S->qld[rs.q],
+      lp_add_moves(lp, a * (int)lab4.size() + b, S->qbase[rs.q] + rs.off + (long long)S->qld[rs.q] * cs.off, S->qld[rs.q],
                    rs.dim, rs.dim_pad, cs.dim, md.mb, md.me);
     }
   for (const MoveSrc& m : S->msrc) {
@@ -372,7 +390,7 @@ int sec_build(dmrg2d_ops* ops, const dmrg2d_block* L, const dmrg2d_block* R, con
     if (gs == DMRG2D_OK) {
       S->gp_ok = true;
       ops->tc_ok = 1;
-      for (int p = 0; p < 4; ++p) ops->tc_cfg[p] = 5;  // 128 x 256 longest-first
+      for (int p = 0; p < 4; ++p) ops->tc_cfg[p] = default_cfg(&g, p);
     } else if (gs == DMRG2D_EUNSUPPORTED) {
       clear_error();  // CUDA-core path only for this sector structure
     } else {
@@ -395,6 +413,12 @@ int sec_apply(const dmrg2d_ops* ops, const void* v, void* y, int precision, cuda
   const SecState* S = (const SecState*)ops->sec;
   if (!S) return set_error(DMRG2D_EINVAL, "not a sector-restricted ops object");
   const LongPlan* lp = ops->lp;
+  // tensor-core configuration; the segment kernels store Y in 16-byte pieces, so unless they
+  // were asked for, a Y off that boundary takes the grouped kernel
+  const int tp = precision == DMRG2D_TF32 ? DMRG2D_TF32 : DMRG2D_BF16;
+  int cfg = ops->tc_cfg[tp];
+  if (cfg == 2 * gp_num_configs() && !ops->tc_chosen[tp] && ((uintptr_t)y & 15) != 0)
+    cfg = grouped_cfg(tp);
   // timed kernel: the block products here; the grouped tensor-core launch times itself
   const bool simt =
       precision == DMRG2D_FP64 || precision == DMRG2D_FP32 || precision == DMRG2D_FP64X;
@@ -412,7 +436,7 @@ int sec_apply(const dmrg2d_ops* ops, const void* v, void* y, int precision, cuda
     D2_TRY(lp_launch_f32(lp, (const float*)v, (float*)y, s));
     if (ev.second) D2_CUDA(cudaEventRecord(ev.second, s));
     D2_TRY(lp_moves_f32(lp, (const float*)v, (float*)y, s));
-  } else if (precision == DMRG2D_BF16X3 && S->gp_ok && ops->tc_cfg[DMRG2D_BF16] == 2 * gp_num_configs()) {
+  } else if (precision == DMRG2D_BF16X3 && S->gp_ok && cfg == 2 * gp_num_configs()) {
     // segment kernels: three products, then the moves on v_hi and v_lo
     const __nv_bfloat16* vhi = (const __nv_bfloat16*)v;
     const __nv_bfloat16* vlo = vhi + ops->n_vec;
@@ -422,19 +446,17 @@ int sec_apply(const dmrg2d_ops* ops, const void* v, void* y, int precision, cuda
     D2_TRY(lp_moves_bf16(lp, vhi, (float*)y, s));
     D2_TRY(lp_moves_bf16(lp, vlo, (float*)y, s));
   } else if ((precision == DMRG2D_TF32 || precision == DMRG2D_BF16) && S->gp_ok &&
-             ops->tc_cfg[precision] == 2 * gp_num_configs()) {
+             cfg == 2 * gp_num_configs()) {
     // segment kernels (M along the long dimension of each V_q), then the scalar moves
     D2_TRY(gp_launch_seg(ops, &S->plan, v, (float*)y, precision, s));
-    {
-      if (precision == DMRG2D_BF16)
-        D2_TRY(lp_moves_bf16(lp, (const __nv_bfloat16*)v, (float*)y, s));
-      else
-        D2_TRY(lp_moves_f32(lp, (const float*)v, (float*)y, s));
-    }
+    if (precision == DMRG2D_BF16)
+      D2_TRY(lp_moves_bf16(lp, (const __nv_bfloat16*)v, (float*)y, s));
+    else
+      D2_TRY(lp_moves_f32(lp, (const float*)v, (float*)y, s));
   } else if (precision == DMRG2D_BF16X3 && S->gp_ok) {
     // v = [v_hi | v_lo]: H_hi v_hi + H_hi v_lo + H_lo v_hi with the layout chosen for BF16,
     // the scalar moves applied to v_hi and v_lo (in the epilogues, or their own kernel)
-    const int G = gp_num_configs(), cfg = ops->tc_cfg[DMRG2D_BF16];
+    const int G = gp_num_configs();
     const bool fused = cfg < G;
     const __nv_bfloat16* vhi = (const __nv_bfloat16*)v;
     const __nv_bfloat16* vlo = vhi + ops->n_vec;
@@ -448,7 +470,7 @@ int sec_apply(const dmrg2d_ops* ops, const void* v, void* y, int precision, cuda
   } else if ((precision == DMRG2D_TF32 || precision == DMRG2D_BF16) && S->gp_ok) {
     // tc_cfg < G: one launch, the grouped kernel's epilogue adds the scalar moves;
     // G <= tc_cfg < 2G: the moves run in their own kernel after it (G tile layouts)
-    const int G = gp_num_configs(), cfg = ops->tc_cfg[precision];
+    const int G = gp_num_configs();
     const bool fused = cfg < G;
     D2_TRY(gp_launch(ops, &S->plan, v, (float*)y, precision, cfg % G, s, fused));
     if (!fused) {
