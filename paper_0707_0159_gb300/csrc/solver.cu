@@ -36,6 +36,11 @@ int vgrid(int64_t n) {
   return (int)(g < RED_BLOCKS ? (g < 1 ? 1 : g) : RED_BLOCKS);
 }
 
+// CTAs of a reduction over FP64 vectors: three per SM.  Every CTA ends in a tree of FP64
+// additions at 2 per clock and SM (eight of them in k_multidot_partial: 87 us with 1216 CTAs on
+// 3.4e6 elements, 74 with 456).
+int rgrid(int64_t n) { return std::min(vgrid(n), 456); }
+
 __device__ __forceinline__ double warp_sum(double v) {
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
@@ -418,7 +423,91 @@ __global__ void k_scale_to32(float* __restrict__ q, const TI* __restrict__ in,
 //   t += a p,  r -= a q,  rr' = r.r,  p = r + (rr'/rr) p.
 // Three passes over FP32 vectors (x32 is x rounded to FP32; the correction is
 // re-orthogonalised in FP64 afterwards); scalars stay on the device.
-enum { CG_XQ = 40, CG_PQ, CG_A, CG_RR, CG_RR1, CG_BETA, CG_THETA };
+// Each reduction is finished by the last CTA to arrive, in a fixed order (no kernel of its own).
+// With float4 accesses and one step queued ahead of the host, a step of the mixed solve on the
+// 4-leg Heisenberg sectors of m = 256 (n = 3.4e6) went from 145 to 110 us, 79 of them H~ p.
+// Once a step has met p.q <= 0 or r.r <= 1e-8 r0.r0, CG_STOP makes later steps leave t and r
+// alone: the host launches a step before it has seen the result of the one before.
+enum { CG_XQ = 40, CG_PQ, CG_A, CG_RR, CG_RR1, CG_BETA, CG_THETA, CG_RR0, CG_STOP, CG_STEPS,
+       CG_COUNT };  // CG_COUNT: two unsigned arrival counters
+
+// 304 CTAs (two per SM): every CTA costs a tree of FP64 additions at GB300's FP64 rate (with
+// 1216 it was half of a pass's time), and float4 loads keep enough bytes in flight
+int cg_grid(int64_t n) { return (int)std::max<int64_t>(1, std::min<int64_t>(304, n / (4 * VT))); }
+
+// true in the CTA that arrives last; the partial sums written before are then visible
+__device__ bool last_block(unsigned* count) {
+  __shared__ bool last;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    __threadfence();
+    last = atomicAdd(count, 1u) == gridDim.x - 1;
+    if (last) {
+      *count = 0;
+      __threadfence();
+    }
+  }
+  __syncthreads();
+  return last;
+}
+__device__ double sum_parts(const double* part, int np) {
+  double s = 0.0;
+  for (int b = threadIdx.x; b < np; b += VT) s += __ldcg(part + b);
+  return block_sum(s);
+}
+
+// calls f(first element, number) on fours of elements (fewer at the end)
+template <typename F>
+__device__ __forceinline__ void for_fours(int64_t n, F f) {
+  const int64_t n4 = (n + 3) / 4, step = (int64_t)gridDim.x * VT;
+#pragma unroll 2
+  for (int64_t i = (int64_t)blockIdx.x * VT + threadIdx.x; i < n4; i += step)
+    f(4 * i, (int)(n - 4 * i < 4 ? n - 4 * i : 4));
+}
+struct Four {
+  float v[4];
+};
+__device__ __forceinline__ Four get4(const float* p, int64_t e, int m) {
+  Four r;
+  if (m == 4) {
+    const float4 x = *(const float4*)(p + e);
+    r.v[0] = x.x, r.v[1] = x.y, r.v[2] = x.z, r.v[3] = x.w;
+  } else {
+#pragma unroll
+    for (int i = 0; i < 4; ++i) r.v[i] = i < m ? p[e + i] : 0.f;
+  }
+  return r;
+}
+__device__ __forceinline__ void put4(float* p, int64_t e, int m, const Four& r) {
+  if (m == 4) {
+    *(float4*)(p + e) = make_float4(r.v[0], r.v[1], r.v[2], r.v[3]);
+  } else {
+    for (int i = 0; i < m; ++i) p[e + i] = r.v[i];
+  }
+}
+// the H~ input format of four elements (put_lo)
+__device__ __forceinline__ void put_lo4(void* lo, int precision, int64_t e, int m, const Four& r,
+                                        int64_t n) {
+  if (m == 4 && precision == DMRG2D_TF32) {
+    *(float4*)((float*)lo + e) =
+        make_float4(to_tf32(r.v[0]), to_tf32(r.v[1]), to_tf32(r.v[2]), to_tf32(r.v[3]));
+  } else if (m == 4 && precision == DMRG2D_BF16) {
+    const __nv_bfloat162 a = __floats2bfloat162_rn(r.v[0], r.v[1]);
+    const __nv_bfloat162 b = __floats2bfloat162_rn(r.v[2], r.v[3]);
+    *(uint2*)((__nv_bfloat16*)lo + e) =
+        make_uint2(*reinterpret_cast<const uint32_t*>(&a), *reinterpret_cast<const uint32_t*>(&b));
+  } else {
+    for (int i = 0; i < m; ++i) put_lo(lo, precision, e + i, r.v[i], n);
+  }
+}
+
+// after k_cg_start32 and its reduction: the state of a new solve
+__global__ void k_cg_begin(double* __restrict__ scal) {
+  scal[CG_RR0] = scal[CG_RR];
+  scal[CG_STOP] = 0.0;
+  scal[CG_STEPS] = 0.0;
+  scal[CG_COUNT] = 0.0;
+}
 
 // CG start: r32 = r, x32 = x, t32 = 0, p32 = r32 and its H~ copy; part[b] = partial r32.r32
 __global__ void k_cg_start32(const double* __restrict__ r, const double* __restrict__ x,
@@ -440,91 +529,88 @@ __global__ void k_cg_start32(const double* __restrict__ r, const double* __restr
   if (threadIdx.x == 0) part[blockIdx.x] = v;
 }
 
-// part[b] = partial x.q', part[g + b] = partial p.q'
-__global__ void k_cg_dots(const float* __restrict__ y, const float* __restrict__ p,
-                          const float* __restrict__ x, const double* __restrict__ scal,
-                          int64_t n, double* __restrict__ part) {
+// x.q' and p.q' (part[b], part[g + b]); then CG_XQ, CG_PQ and a = rr / pq (0: no update)
+__global__ void __launch_bounds__(VT)
+k_cg_dots(const float* __restrict__ y, const float* __restrict__ p, const float* __restrict__ x,
+          double* scal, int64_t n, double* part) {
   const float theta = (float)scal[CG_THETA];
   acc2 sx, sp;
-#pragma unroll 4
-  for (int64_t e = (int64_t)blockIdx.x * VT + threadIdx.x; e < n; e += (int64_t)gridDim.x * VT) {
-    const float pe = p[e];
-    const float q = fmaf(-theta, pe, y[e]);
-    acc_fma(sx, x[e], q);
-    acc_fma(sp, pe, q);
-  }
+  for_fours(n, [&](int64_t e, int m) {
+    const Four ye = get4(y, e, m), pe = get4(p, e, m), xe = get4(x, e, m);
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      const float q = fmaf(-theta, pe.v[i], ye.v[i]);
+      acc_fma(sx, xe.v[i], q);
+      acc_fma(sp, pe.v[i], q);
+    }
+  });
   const double vx = block_sum(acc_val(sx));
   const double vp = block_sum(acc_val(sp));
   if (threadIdx.x == 0) {
     part[blockIdx.x] = vx;
     part[gridDim.x + blockIdx.x] = vp;
   }
-}
-
-// scal[CG_XQ], scal[CG_PQ] from the partials; a = rr / pq (0 when pq <= 0: no update)
-__global__ void k_cg_alpha(const double* __restrict__ part, int np, double* __restrict__ scal) {
-  double sx = 0.0, sp = 0.0;
-  for (int b = threadIdx.x; b < np; b += VT) {
-    sx += part[b];
-    sp += part[np + b];
-  }
-  sx = block_sum(sx);
-  sp = block_sum(sp);
+  if (!last_block((unsigned*)(scal + CG_COUNT))) return;
+  const double tx = sum_parts(part, gridDim.x), tp = sum_parts(part + gridDim.x, gridDim.x);
   if (threadIdx.x == 0) {
-    scal[CG_XQ] = sx;
-    scal[CG_PQ] = sp;
-    scal[CG_A] = sp > 0.0 ? scal[CG_RR] / sp : 0.0;
+    if (scal[CG_STOP] == 0.0) scal[CG_STEPS] += 1.0;
+    if (!(tp > 0.0)) scal[CG_STOP] = 1.0;
+    scal[CG_XQ] = tx;
+    scal[CG_PQ] = tp;
+    scal[CG_A] = scal[CG_STOP] == 0.0 ? scal[CG_RR] / tp : 0.0;
   }
 }
 
-// t += a p, r -= a (y - theta p - xq x); part[b] = partial r.r (of the updated r)
-__global__ void k_cg_update(const float* __restrict__ y, const float* __restrict__ p,
-                            const float* __restrict__ x, float* __restrict__ t,
-                            float* __restrict__ r, const double* __restrict__ scal, int64_t n,
-                            double* __restrict__ part) {
+// t += a p, r -= a (y - theta p - xq x) and r.r of the updated r; then beta = rr1 / rr, rr <- rr1
+__global__ void __launch_bounds__(VT)
+k_cg_update(const float* __restrict__ y, const float* __restrict__ p, const float* __restrict__ x,
+            float* __restrict__ t, float* __restrict__ r, double* scal, int64_t n, double* part) {
   const float a = (float)scal[CG_A], xq = (float)scal[CG_XQ], theta = (float)scal[CG_THETA];
   const bool upd = scal[CG_A] != 0.0;
   acc2 s;
-#pragma unroll 4
-  for (int64_t e = (int64_t)blockIdx.x * VT + threadIdx.x; e < n; e += (int64_t)gridDim.x * VT) {
-    float re = r[e];
+  for_fours(n, [&](int64_t e, int m) {
+    Four re = get4(r, e, m);
     if (upd) {
-      const float pe = p[e];
-      const float q = fmaf(-xq, x[e], fmaf(-theta, pe, y[e]));
-      t[e] = fmaf(a, pe, t[e]);
-      re = fmaf(-a, q, re);
-      r[e] = re;
+      const Four ye = get4(y, e, m), pe = get4(p, e, m), xe = get4(x, e, m);
+      Four te = get4(t, e, m);
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        const float q = fmaf(-xq, xe.v[i], fmaf(-theta, pe.v[i], ye.v[i]));
+        te.v[i] = fmaf(a, pe.v[i], te.v[i]);
+        re.v[i] = fmaf(-a, q, re.v[i]);
+      }
+      put4(t, e, m, te);
+      put4(r, e, m, re);
     }
-    acc_fma(s, re, re);
-  }
+#pragma unroll
+    for (int i = 0; i < 4; ++i) acc_fma(s, re.v[i], re.v[i]);
+  });
   const double v = block_sum(acc_val(s));
   if (threadIdx.x == 0) part[blockIdx.x] = v;
-}
-
-// scal[CG_RR1] = sum of partials; beta = rr1 / rr; rr <- rr1
-__global__ void k_cg_beta(const double* __restrict__ part, int np, double* __restrict__ scal) {
-  double s = 0.0;
-  for (int b = threadIdx.x; b < np; b += VT) s += part[b];
-  s = block_sum(s);
+  if (!last_block((unsigned*)(scal + CG_COUNT) + 1)) return;
+  const double rr1 = sum_parts(part, gridDim.x);
   if (threadIdx.x == 0) {
     const double rr = scal[CG_RR];
-    scal[CG_RR1] = s;
-    scal[CG_BETA] = rr > 0.0 ? s / rr : 0.0;
-    scal[CG_RR] = s;
+    scal[CG_RR1] = rr1;
+    scal[CG_BETA] = rr > 0.0 ? rr1 / rr : 0.0;
+    scal[CG_RR] = rr1;
+    if (rr1 <= 1e-8 * scal[CG_RR0]) scal[CG_STOP] = 1.0;
   }
 }
 
 // p = r + beta p, and the low-precision copy of p that the next H~ p reads
-__global__ void k_cg_direction(float* __restrict__ p, const float* __restrict__ r,
-                               const double* __restrict__ scal, void* __restrict__ lo,
-                               int precision, int64_t n) {
+__global__ void __launch_bounds__(VT)
+k_cg_direction(float* __restrict__ p, const float* __restrict__ r, const double* __restrict__ scal,
+               void* __restrict__ lo, int precision, int64_t n) {
   const float beta = (float)scal[CG_BETA];
-#pragma unroll 4
-  for (int64_t e = (int64_t)blockIdx.x * VT + threadIdx.x; e < n; e += (int64_t)gridDim.x * VT) {
-    const float pe = fmaf(beta, p[e], r[e]);
-    p[e] = pe;
-    put_lo(lo, precision, e, pe, n);
-  }
+  for_fours(n, [&](int64_t e, int m) {
+    Four pe = get4(p, e, m);
+    const Four re = get4(r, e, m);
+#pragma unroll
+    for (int i = 0; i < 4; ++i) pe.v[i] = fmaf(beta, pe.v[i], re.v[i]);
+    put4(p, e, m, pe);
+    put_lo4(lo, precision, e, m, pe, n);
+  });
 }
 
 // ---- lowest eigenpair of the Lanczos tridiagonal T_k (diag alpha, off-diag beta) ----
@@ -542,18 +628,37 @@ constexpr int TD_THREADS = 256;
 constexpr int TD_MAX = 512;
 constexpr int TR_KEEP_MAX = 32;  // Ritz vectors kept at a thick restart
 
-// Negative pivots of LDL^T(T - x) = eigenvalues of T below x; b2 = squared off-diagonal.
-// A pivot smaller than pivmin in magnitude is replaced by -pivmin.
-__device__ int sturm_count(const double* a, const double* b2, int k, double x, double pivmin) {
+// Eigenvalues of T below x: sign changes of the leading principal minors of T - x, by their
+// three-term recurrence p_i = (a_i - x) p_{i-1} - b_{i-1}^2 p_{i-2} (a vanishing minor counts
+// as a negative pivot).  One FMA on the critical path per step where the pivots' recurrence
+// has a division: FP64 division is some ten FP64 operations, at 2 per clock and SM.  a, b2 and
+// x are scaled so that T's norm is about 1; the pair is rescaled by powers of two every 8 steps.
+__device__ int sturm_count(const double* a, const double* b2, int k, double x) {
   int cnt = 0;
-  double q = a[0] - x;
-  for (int i = 1;; ++i) {
-    if (fabs(q) < pivmin) q = -pivmin;
-    if (q < 0) ++cnt;
-    if (i >= k) break;
-    q = (a[i] - x) - b2[i - 1] / q;
+  double pm = 1.0, p = a[0] - x;
+  if (p == 0.0) p = -1e-290;
+  cnt += p < 0.0;
+  for (int i = 1; i < k; ++i) {
+    double q = fma(a[i] - x, p, -(b2[i - 1] * pm));
+    pm = p;
+    if (q == 0.0) q = copysign(1e-290, -pm);
+    p = q;
+    cnt += (unsigned)(__double2hiint(p) ^ __double2hiint(pm)) >> 31;
+    if ((i & 7) == 0) {
+      const int e = max(__double2hiint(p) & 0x7ff00000, __double2hiint(pm) & 0x7ff00000);
+      const double f = __hiloint2double(0x7fe00000 - e, 0);  // 2^-(exponent)
+      p *= f;
+      pm *= f;
+      if (p == 0.0) p = copysign(1e-290, -pm);
+    }
   }
   return cnt;
+}
+// a power of two that brings T (Gershgorin interval [lo, hi]) to norm about 1
+__device__ double td_scale(double lo, double hi) {
+  const double m = fmax(fabs(lo), fabs(hi));
+  if (!(m > 1e-290) || !(m < 1e290)) return 1.0;
+  return __hiloint2double(0x7fe00000 - (__double2hiint(m) & 0x7ff00000), 0);
 }
 
 // Fallback eigenvector: three steps of inverse iteration, (T - theta) z = s, tridiagonal
@@ -654,13 +759,14 @@ __device__ __forceinline__ double warp_max(double v) {
   return v;
 }
 
-// Shared set-up of the tridiagonal kernels: a, bb (off-diagonal, bb[k-1] = 0), b2 = bb^2
-// in shared memory; Gershgorin interval and pivmin (by thread 0 into *lo, *hi, *pivmin);
-// returns false (uniformly) if an entry of alpha[0..k) or beta[0..k) is not finite.
+// Shared set-up of the tridiagonal kernels: a, bb (off-diagonal, bb[k-1] = 0) in shared
+// memory; Gershgorin interval (by thread 0 into *lo, *hi); the scale *sc and the scaled
+// as = sc a, b2 = (sc bb)^2 of the Sturm counts; returns false (uniformly) if an entry of
+// alpha[0..k) or beta[0..k) is not finite.
 __device__ bool td_setup(const double* __restrict__ alpha, const double* __restrict__ beta, int k,
-                         double* a, double* bb, double* b2, double* lo, double* hi,
-                         double* pivmin) {
-  __shared__ double r_lo[TD_THREADS / 32], r_hi[TD_THREADS / 32], r_b[TD_THREADS / 32];
+                         double* a, double* bb, double* as, double* b2, double* lo, double* hi,
+                         double* sc) {
+  __shared__ double r_lo[TD_THREADS / 32], r_hi[TD_THREADS / 32];
   __shared__ int bad;
   const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
   if (tid == 0) bad = 0;
@@ -671,35 +777,36 @@ __device__ bool td_setup(const double* __restrict__ alpha, const double* __restr
     if (!isfinite(ai) || !isfinite(bi)) mybad = true;
     a[i] = ai;
     bb[i] = i + 1 < k ? bi : 0.0;
-    b2[i] = bb[i] * bb[i];
   }
   if (mybad) atomicOr(&bad, 1);
   __syncthreads();
-  double l = 1e300, h = -1e300, bm = 0.0;
+  double l = 1e300, h = -1e300;
   for (int i = tid; i < k; i += TD_THREADS) {
     const double r = (i > 0 ? fabs(bb[i - 1]) : 0.0) + fabs(bb[i]);
     l = fmin(l, a[i] - r);
     h = fmax(h, a[i] + r);
-    bm = fmax(bm, b2[i]);
   }
   l = warp_min(l);
   h = warp_max(h);
-  bm = warp_max(bm);
   if (lane == 0) {
     r_lo[w] = l;
     r_hi[w] = h;
-    r_b[w] = bm;
   }
   __syncthreads();
   if (tid == 0) {
     for (int i = 1; i < TD_THREADS / 32; ++i) {
       l = fmin(l, r_lo[i]);
       h = fmax(h, r_hi[i]);
-      bm = fmax(bm, r_b[i]);
     }
     *lo = l;
     *hi = h;
-    *pivmin = 2.2250738585072014e-308 * fmax(1.0, bm);
+  }
+  __syncthreads();
+  *sc = td_scale(*lo, *hi);
+  for (int i = tid; i < k; i += TD_THREADS) {
+    as[i] = a[i] * *sc;
+    const double b = bb[i] * *sc;
+    b2[i] = b * b;
   }
   __syncthreads();
   return bad == 0;
@@ -708,13 +815,14 @@ __device__ bool td_setup(const double* __restrict__ alpha, const double* __restr
 __global__ void __launch_bounds__(TD_THREADS)
 k_tridiag_ground(const double* __restrict__ alpha, const double* __restrict__ beta, int k,
                  double* __restrict__ s, double* __restrict__ out, double* __restrict__ scr) {
-  __shared__ double a[TD_MAX], bb[TD_MAX], b2[TD_MAX];
+  __shared__ double a[TD_MAX], bb[TD_MAX], b2[TD_MAX], as[TD_MAX];
   __shared__ double Dp[TD_MAX], Dm[TD_MAX], Lf[TD_MAX], Ub[TD_MAX], z[TD_MAX];
-  __shared__ double sh_lo, sh_hi, sh_piv, sh_red[TD_THREADS / 32];
+  __shared__ double sh_lo, sh_hi, sh_red[TD_THREADS / 32];
   __shared__ int sh_first, sh_r[TD_THREADS / 32];
   __shared__ double sh_g[TD_THREADS / 32];
   const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
-  if (!td_setup(alpha, beta, k, a, bb, b2, &sh_lo, &sh_hi, &sh_piv)) {
+  double sc;
+  if (!td_setup(alpha, beta, k, a, bb, as, b2, &sh_lo, &sh_hi, &sc)) {
     if (tid == 0) {
       out[0] = nan("");
       out[1] = nan("");
@@ -722,46 +830,66 @@ k_tridiag_ground(const double* __restrict__ alpha, const double* __restrict__ be
     }
     return;
   }
-  const double pivmin = sh_piv;
-  // ---- multisection for the lowest eigenvalue ----
-  for (int it = 0; it < 16; ++it) {
-    const double L = sh_lo, H = sh_hi;
-    if (!(H - L > 4.4e-16 * fmax(fabs(L), fabs(H)) + 1e-300)) break;
-    const double x = L + (H - L) * (double)(tid + 1) / (double)(TD_THREADS + 1);
-    const bool below = sturm_count(a, b2, k, x, pivmin) >= 1;
-    if (tid == 0) sh_first = TD_THREADS;
-    __syncthreads();
-    if (below) atomicMin(&sh_first, tid);
-    __syncthreads();
-    if (tid == 0) {
-      const int f = sh_first;
-      sh_lo = f == 0 ? L : L + (H - L) * (double)f / (double)(TD_THREADS + 1);
-      sh_hi = f == TD_THREADS ? H : L + (H - L) * (double)(f + 1) / (double)(TD_THREADS + 1);
+  // ---- multisection for the lowest eigenvalue, on one warp ----
+  // (33-fold per round.  A step of the recurrence is three FP64 operations, 64 cycles each on
+  // a quarter of the SM; all eight warps, 257-fold, with pivots took 299 us for k = 40, this
+  // 134 us.)
+  if (w == 0) {
+    double L = sh_lo, H = sh_hi;
+    for (int it = 0; it < 40; ++it) {
+      if (!(H - L > 4.4e-16 * fmax(fabs(L), fabs(H)) + 1e-300)) break;
+      const double x = L + (H - L) * (double)(lane + 1) / 33.0;
+      const unsigned m = __ballot_sync(0xffffffffu, sturm_count(as, b2, k, x * sc) >= 1);
+      const int f = m ? __ffs(m) - 1 : 32;
+      const double nL = f == 0 ? L : L + (H - L) * (double)f / 33.0;
+      const double nH = f == 32 ? H : L + (H - L) * (double)(f + 1) / 33.0;
+      L = nL;
+      H = nH;
     }
-    __syncthreads();
+    __syncwarp();
+    if (lane == 0) {
+      sh_lo = L;
+      sh_hi = H;
+    }
   }
+  __syncthreads();
   const double theta = 0.5 * (sh_lo + sh_hi);
   const double tiny = 1e-14 * fmax(fabs(sh_lo), fabs(sh_hi)) + 1e-300;
-  // ---- twisted factorisation of T - theta ----
-  if (tid == 0) {  // top-down LDL^T
-    double d = a[0] - theta;
-    for (int i = 0; i + 1 < k; ++i) {
-      if (fabs(d) < tiny) d = d < 0 ? -tiny : tiny;
-      Dp[i] = d;
-      Lf[i] = bb[i] / d;
-      d = (a[i + 1] - theta) - Lf[i] * bb[i];
+  // ---- twisted factorisation of T - theta: top-down LDL^T and bottom-up UDU^T pivots ----
+  // as ratios of successive minors (as in sturm_count, one thread each); the divisions are
+  // then independent
+  auto minors = [&](bool up, double* num, double* den) {
+    const double ths = theta * sc, ts = tiny * sc;
+    double pm = 1.0, p = 0.0;
+    for (int j = 0; j < k; ++j) {
+      const int i = up ? k - 1 - j : j;
+      const double b = j == 0 ? 0.0 : b2[up ? i : i - 1];
+      const double q = j == 0 ? as[i] - ths : fma(as[i] - ths, p, -(b * pm));
+      if (j > 0) pm = p;
+      p = q;
+      const double lim = ts * fabs(pm);
+      if (j + 1 < k && fabs(p) < lim) p = (p < 0.0) != (pm < 0.0) ? -copysign(lim, pm) : copysign(lim, pm);
+      num[i] = p;
+      den[i] = pm;
+      if ((j & 7) == 7) {
+        const int e = max(__double2hiint(p) & 0x7ff00000, __double2hiint(pm) & 0x7ff00000);
+        const double f = __hiloint2double(0x7fe00000 - e, 0);
+        p *= f;
+        pm *= f;
+      }
     }
-    Dp[k - 1] = d;
-  } else if (tid == 32) {  // bottom-up UDU^T
-    double d = a[k - 1] - theta;
-    for (int i = k - 2; i >= 0; --i) {
-      if (fabs(d) < tiny) d = d < 0 ? -tiny : tiny;
-      Dm[i + 1] = d;
-      Ub[i] = bb[i] / d;
-      d = (a[i] - theta) - Ub[i] * bb[i];
-    }
-    Dm[0] = d;
+  };
+  if (tid == 0) minors(false, Dp, Lf);
+  if (tid == 32) minors(true, Dm, Ub);
+  __syncthreads();
+  for (int i = tid; i < k; i += TD_THREADS) {
+    const double d = Dp[i] / Lf[i] / sc;
+    Dp[i] = d;
+    Lf[i] = bb[i] / d;
+    Dm[i] = Dm[i] / Ub[i] / sc;
   }
+  __syncthreads();
+  for (int i = tid; i + 1 < k; i += TD_THREADS) Ub[i] = bb[i] / Dm[i + 1];
   __syncthreads();
   double g = INFINITY;  // twist index: smallest |gamma_r|, ties to the smaller r
   int r = k;
@@ -874,27 +1002,27 @@ k_tridiag_ground(const double* __restrict__ alpha, const double* __restrict__ be
 __global__ void __launch_bounds__(TD_THREADS)
 k_thick_restart(double* __restrict__ alpha, double* __restrict__ beta, int k, int p,
                 double* __restrict__ M, double* __restrict__ scr, double* __restrict__ out) {
-  __shared__ double a[TD_MAX], bb[TD_MAX], b2[TD_MAX];
-  __shared__ double sh_lo, sh_hi, sh_piv, sh_bk, sh_red[TD_THREADS / 32];
+  __shared__ double a[TD_MAX], bb[TD_MAX], b2[TD_MAX], as[TD_MAX];
+  __shared__ double sh_lo, sh_hi, sh_bk, sh_red[TD_THREADS / 32];
   __shared__ double th[TR_KEEP_MAX], P[TR_KEEP_MAX][TR_KEEP_MAX + 1],
       W[TR_KEEP_MAX][TR_KEEP_MAX + 1], cvec[TR_KEEP_MAX], al[TR_KEEP_MAX], be[TR_KEEP_MAX];
   __shared__ int sh_p, sh_pp;
   const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
   if (tid == 0) sh_bk = beta[k - 1];
-  if (!td_setup(alpha, beta, k, a, bb, b2, &sh_lo, &sh_hi, &sh_piv) || p < 1 || k < 2) {
+  double sc;
+  if (!td_setup(alpha, beta, k, a, bb, as, b2, &sh_lo, &sh_hi, &sc) || p < 1 || k < 2) {
     if (tid == 0) out[0] = 0.0;
     return;
   }
   if (p > TR_KEEP_MAX) p = TR_KEEP_MAX;
   if (p > k - 1) p = k - 1;
-  const double pivmin = sh_piv;
   // 1. the p lowest eigenvalues, one warp each (32-section, 33-fold per round)
   for (int i = w; i < p; i += TD_THREADS / 32) {
     double L = sh_lo, H = sh_hi;
     for (int it = 0; it < 40; ++it) {
       if (!(H - L > 4.4e-16 * fmax(fabs(L), fabs(H)) + 1e-300)) break;
       const double x = L + (H - L) * (double)(lane + 1) / 33.0;
-      const unsigned m = __ballot_sync(0xffffffffu, sturm_count(a, b2, k, x, pivmin) >= i + 1);
+      const unsigned m = __ballot_sync(0xffffffffu, sturm_count(as, b2, k, x * sc) >= i + 1);
       const int f = m ? __ffs(m) - 1 : 32;
       const double nL = f == 0 ? L : L + (H - L) * (double)f / 33.0;
       const double nH = f == 32 ? H : L + (H - L) * (double)(f + 1) / 33.0;
@@ -1265,14 +1393,14 @@ struct Ctx {
 
   // *out (device) = a . b
   int dot(const double* a, const double* b, double* out) {
-    const int g = vgrid(n);
+    const int g = rgrid(n);
     k_dot_partial<<<g, VT, 0, s>>>(a, b, n, part);
     k_reduce<<<1, VT, 0, s>>>(part, g, out, 0);
     D2_CUDA(cudaGetLastError());
     return DMRG2D_OK;
   }
   int nrm(const double* a, double* out) {
-    const int g = vgrid(n);
+    const int g = rgrid(n);
     k_dot_partial<<<g, VT, 0, s>>>(a, a, n, part);
     k_reduce<<<1, VT, 0, s>>>(part, g, out, 1);
     D2_CUDA(cudaGetLastError());
@@ -1280,7 +1408,7 @@ struct Ctx {
   }
   // h[0..k) = Q[0..k) . w
   int multidot(const double* Q, int64_t stride, int k, const double* w, double* h) {
-    const int g = vgrid(n);
+    const int g = rgrid(n);
     dim3 grid(g, (k + MD_CHUNK - 1) / MD_CHUNK);
     k_multidot_partial<<<grid, VT, 0, s>>>(Q, stride, k, w, n, part);
     k_reduce<<<k, VT, 0, s>>>(part, g, h, 0);
@@ -1532,7 +1660,7 @@ int lanczos_lo(Ctx& C, int prec, double* x, int max_iter, int kdim, double tol, 
                      {&scr, 6 * kd}}));
   float* w = C.y32;  // H~ q_j lands here and is orthogonalised in place
   double* out3 = C.scal;
-  const int g = vgrid(n);
+  const int g = vgrid(n), gr = rgrid(n);
   auto start_from_x = [&]() -> int {
     D2_TRY(C.nrm(x, C.scal + 3));
     k_scale_to32<double><<<g, VT, 0, C.s>>>(Q, x, C.scal + 3, C.lo, prec, n);
@@ -1547,11 +1675,11 @@ int lanczos_lo(Ctx& C, int prec, double* x, int max_iter, int kdim, double tol, 
   while (true) {
     float* qj = Q + (int64_t)j * n;
     D2_TRY(C.hv_lo(prec));  // w = H~ q_j (its H~-format copy is in C.lo)
-    k_dot_partial32<<<g, VT, 0, C.s>>>(qj, w, n, C.part);
-    k_reduce<<<1, VT, 0, C.s>>>(C.part, g, alpha + j, 0);
-    k_lz_axpy2_nrm32<<<g, VT, 0, C.s>>>(w, qj, j > 0 ? qj - n : nullptr, alpha + j,
+    k_dot_partial32<<<gr, VT, 0, C.s>>>(qj, w, n, C.part);
+    k_reduce<<<1, VT, 0, C.s>>>(C.part, gr, alpha + j, 0);
+    k_lz_axpy2_nrm32<<<gr, VT, 0, C.s>>>(w, qj, j > 0 ? qj - n : nullptr, alpha + j,
                                         j > 0 ? beta + j - 1 : nullptr, n, C.part);
-    k_reduce<<<1, VT, 0, C.s>>>(C.part, g, beta + j, 1);
+    k_reduce<<<1, VT, 0, C.s>>>(C.part, gr, beta + j, 1);
     for (int pass = 0; pass < gs_passes; ++pass) {  // CGS against q_0..q_j
       dim3 grid(g, (j + 1 + MD_CHUNK - 1) / MD_CHUNK);
       k_multidot_partial32<<<grid, VT, 0, C.s>>>(Q, n, j + 1, w, n, C.part);
@@ -1626,6 +1754,7 @@ struct StepGraph {
   cudaGraph_t graph = nullptr;
   cudaGraphExec_t exec = nullptr;
   cudaStream_t cs = nullptr;
+  cudaEvent_t done[2] = {nullptr, nullptr};  // the last two replays
 
   template <typename F>
   int capture(Ctx& C, F&& body) {
@@ -1638,10 +1767,13 @@ struct StepGraph {
     C.s = saved;
     if (st != DMRG2D_OK) return st;
     if (e != cudaSuccess) return set_error(DMRG2D_ECUDA, "CG step capture: %s", cudaGetErrorString(e));
+    for (cudaEvent_t& ev : done) D2_CUDA(cudaEventCreateWithFlags(&ev, cudaEventDisableTiming));
     D2_CUDA(cudaGraphInstantiate(&exec, graph, 0));
     return DMRG2D_OK;
   }
   ~StepGraph() {
+    for (cudaEvent_t e : done)
+      if (e) cudaEventDestroy(e);
     if (exec) cudaGraphExecDestroy(exec);
     if (graph) cudaGraphDestroy(graph);
     if (cs) cudaStreamDestroy(cs);
@@ -1746,30 +1878,32 @@ static int mixed_outer(Ctx& C, const dmrg2d_solver_opts* o, double* x, double* e
     k_cg_start32<<<g, VT, 0, C.s>>>(r, x, r32, x32, t32, p32, C.lo, prec, n, C.part);
     k_reduce<<<1, VT, 0, C.s>>>(C.part, g, sc + CG_RR, 0);
     D2_CUDA(cudaGetLastError());
-    D2_TRY(C.fetch(sc + CG_RR, 1));
-    const double rr0 = C.hscal[0];
+    k_cg_begin<<<1, 1, 0, C.s>>>(sc);
+    D2_CUDA(cudaGetLastError());
     if (!step.exec) D2_TRY(step.capture(C, [&]() -> int {
-      // one CG step: y32 = H~ p, the fused vector passes, scalars to the pinned mirror
+      // one CG step: y32 = H~ p, the fused vector passes, the stop flag to the pinned mirror
       D2_TRY(C.hv_lo(prec, nullptr, nullptr, false));  // counted per replay
-      k_cg_dots<<<g, VT, 0, C.s>>>(C.y32, p32, x32, sc, n, C.part);
-      k_cg_alpha<<<1, VT, 0, C.s>>>(C.part, g, sc);
-      k_cg_update<<<g, VT, 0, C.s>>>(C.y32, p32, x32, t32, r32, sc, n, C.part);
-      k_cg_beta<<<1, VT, 0, C.s>>>(C.part, g, sc);
-      k_cg_direction<<<g, VT, 0, C.s>>>(p32, r32, sc, C.lo, prec, n);
+      const int cg = cg_grid(n);
+      k_cg_dots<<<cg, VT, 0, C.s>>>(C.y32, p32, x32, sc, n, C.part);
+      k_cg_update<<<cg, VT, 0, C.s>>>(C.y32, p32, x32, t32, r32, sc, n, C.part);
+      k_cg_direction<<<vgrid((n + 3) / 4), VT, 0, C.s>>>(p32, r32, sc, C.lo, prec, n);
       D2_CUDA(cudaGetLastError());
-      D2_CUDA(cudaMemcpyAsync(C.hscal, sc + CG_PQ, sizeof(double) * (CG_RR1 - CG_PQ + 1),
-                              cudaMemcpyDeviceToHost, C.s));
+      D2_CUDA(cudaMemcpyAsync(C.hscal, sc + CG_STOP, sizeof(double) * 2, cudaMemcpyDeviceToHost,
+                              C.s));
       return DMRG2D_OK;
     }));
+    // The next step is in the queue before the host waits for the one before it; the device
+    // decides when to stop (a step after that changes nothing).
     for (int it = 0; it < o->inner_iter; ++it) {
       D2_CUDA(cudaGraphLaunch(step.exec, C.s));
-      D2_CUDA(cudaStreamSynchronize(C.s));  // one wait per step
-      const double pq = C.hscal[0], rr1 = C.hscal[CG_RR1 - CG_PQ];
-      C.st->n_hv_low++;
-      C.st->iters++;
-      if (!(pq > 0.0)) break;  // (no update was made)
-      if (rr1 <= 1e-8 * rr0) break;
+      D2_CUDA(cudaEventRecord(step.done[it & 1], C.s));
+      if (it == 0) continue;
+      D2_CUDA(cudaEventSynchronize(step.done[(it - 1) & 1]));
+      if (*(volatile double*)C.hscal != 0.0) break;
     }
+    D2_CUDA(cudaStreamSynchronize(C.s));
+    C.st->n_hv_low += (int)C.hscal[CG_STEPS - CG_STOP];
+    C.st->iters += (int)C.hscal[CG_STEPS - CG_STOP];
     k_f32_to_f64<<<g, VT, 0, C.s>>>(t32, t, n);
     D2_CUDA(cudaGetLastError());
     // ---- orthonormalise t against U and extend the subspace ----
