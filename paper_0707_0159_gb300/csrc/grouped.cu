@@ -47,6 +47,12 @@ struct GMaps {
   CUtensorMap vm[GQ_MAX];
 };
 
+// the segment kernels' maps: the operator pool in 32-, 64- and 128-row boxes; the V_q
+struct SMaps {
+  CUtensorMap op[3];
+  CUtensorMap v[GQ_MAX];
+};
+
 struct GParams {
   int ntiles, bn, BK;
   const GTile* tiles;
@@ -87,7 +93,8 @@ struct GDev {
   __nv_bfloat16* pL16lo = nullptr;  // BF16X3: x - bf16(x) rounded to BF16
   __nv_bfloat16* pR16lo = nullptr;
   CUtensorMap mLlo, mRlo[2];
-  CUtensorMap mL32[2], mR32[2], mL32lo, mR32lo;  // the pools in 32-row boxes (segment kernels)
+  // the pools in 32-, 64- and 128-row boxes (segment kernels): [FP32, BF16, BF16 low part]
+  CUtensorMap mLs[3][3], mRs[3][3];
   int KPL = 0, KPR = 0, prL = 0, prR = 0, copies = 1;
   CUtensorMap mL[2], mR[2][2];  // [precision][piece width 128/256]
   int* err = nullptr;
@@ -369,7 +376,8 @@ hv_tc_grouped_kernel(const __grid_constant__ GMaps maps, const GParams p) {
 struct SItem {
   int q, seg, n0, m0;  // matrix; segment (row segment in pass 1, column segment in pass 2);
                        // offset of the N range in the segment; first of the 128 M indices
-  int kb, ke, sdim, pad;  // the segment's operator blocks and extent
+  int kb, ke, sdim;  // the segment's operator blocks and extent
+  int a3;  // pass 2: the V tile in one 3-D box (seg_one_box)
 };
 
 struct SParams {
@@ -385,22 +393,18 @@ struct SParams {
   float* y;
   int* err;
   uint32_t idesc[16][2];  // N = 16 (i + 1); [negate the operator block]
-  uint32_t a2_lbo, a2_sbo, a2_kstep, a2_layout;  // pass 2: MN-major A (as the grouped kernel)
-  int a2_boxes, a2_box_rows;
-  uint32_t a_bytes, b_box_bytes;  // per stage: the A tile; one 32-row box of B
-  int BK, KSTEP;  // K per stage; K per instruction
   int accum_y;    // pass 1: add the Y already stored (BF16X3)
 };
 
 template <int BF16, int PASS>
 __global__ void __launch_bounds__(G_THREADS, 1)
-hv_tc_seg_kernel(const __grid_constant__ GMaps maps, const SParams p) {
+hv_tc_seg_kernel(const __grid_constant__ SMaps maps, const SParams p) {
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = (uint8_t*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
   uint64_t* bars = (uint64_t*)(smem + G_STAGES * G_STAGE);
   uint32_t* tmem_slot = (uint32_t*)(bars + 2 * G_STAGES + 4);
   volatile int* abort = (volatile int*)(tmem_slot + 1);
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = warp_index(), lane = threadIdx.x & 31;
   auto full = [&](int s) { return smem_u32(bars + s); };
   auto empty = [&](int s) { return smem_u32(bars + G_STAGES + s); };
   auto tfull = [&](int b) { return smem_u32(bars + 2 * G_STAGES + b); };
@@ -431,42 +435,49 @@ hv_tc_seg_kernel(const __grid_constant__ GMaps maps, const SParams p) {
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem_base = *tmem_slot;
-  const int BK = p.BK;
+  // K per stage and per instruction; pass 2's A is MN-major, in boxes of A2_ROWS rows (as the
+  // grouped kernel's phase 2)
+  constexpr int BK = BF16 ? 64 : 32, KSTEP = BF16 ? 16 : 8, A2_ROWS = BF16 ? 64 : 32;
 
-  // The operator-block entries of a piece are read by the whole warp, one per lane, and those
-  // of the next piece while this one runs: read one after another by the issuing thread, each
-  // was a global-memory latency in front of the one or two stages of its block (3-leg Hubbard
-  // sectors, m = 1024, TF32 H·v: 3.87 -> 3.44 ms; the two passes now read 9 and 11 GB at 8 TB/s
-  // from L2, a third of it padding of K = 41 to 64).
+  // What bounds the passes is the work of the two role warps between two stages: with loads,
+  // MMAs and stores all left out they took 90 % of their time.  So the operator-block entries
+  // of a piece are read by the whole warp, one per lane, while the piece before runs, pieces
+  // two ahead; the V tile comes in one box and the operator rows in one or two; and the warps'
+  // loop state stays in uniform registers (elect_one).  3-leg Hubbard sectors, m = 1024, TF32:
+  // passes 1160 and 1380 us -> 890 and 875 us, H·v 3.23 -> 2.46 ms; 4-leg Heisenberg sectors,
+  // m = 256: 74.4 -> 60.5 us.
   // {a_pool, b_row, kdim, neg} in pass 1, {a_col, b_pool, kdim, neg} in pass 2
   const int4* const ents = PASS == 0 ? (const int4*)p.k1 : (const int4*)p.k2;
-  const SItem none = {0, 0, 0, 0, 0, 0, 0, 0};
+  auto item = [&](int i) {
+    return i < p.nitems ? p.items[i] : SItem{0, 0, 0, 0, 0, 0, 0, 0};
+  };
   if (warp == 0) {
     // ------------------------------- TMA producer -------------------------------
+    const uint32_t el = elect_one();
     int stage = 0;
     uint32_t phase = 0;
     bool ok = true;
     int ti = blockIdx.x;
-    SItem it = ti < p.nitems ? p.items[ti] : none;
+    SItem it = item(ti), nx = item(ti + gridDim.x);
     int4 ent = it.kb + lane < it.ke ? ents[it.kb + lane] : make_int4(0, 0, 0, 0);
     for (; ti < p.nitems && ok; ti += gridDim.x) {
-      const SItem nx = ti + (int)gridDim.x < p.nitems ? p.items[ti + gridDim.x] : none;
+      const SItem nn = item(ti + 2 * gridDim.x);
       int4 ent_nx = make_int4(0, 0, 0, 0);
       // the operator rows this piece needs, in 32-row boxes (N rounded up to 16 <= 32 nb)
       const int nb = (min(NMAX, it.sdim - it.n0) + 31) / 32;
-      const uint32_t tx = p.a_bytes + (uint32_t)nb * p.b_box_bytes;
-      // lane b copies box b: the V tile's (pass 1: one, rows voff .. (K) by columns m0 .. (M);
-      // pass 2: 32-row boxes of rows m0 .. (M, MN-major) by columns voff .. (K)), then the
-      // operator rows', 32 at a time (the 128B swizzle is a function of the shared-memory
-      // address, so the boxes line up as one tile)
-      const int na = PASS == 0 ? 1 : p.a2_boxes, bi = lane - na;
+      const uint32_t tx = G_STAGE_A + (uint32_t)nb * 32 * 128;
+      // V tile: pass 1 rows voff .. (K) by columns m0 .. (M); pass 2 rows m0 .. (M, MN-major)
+      // by columns voff .. (K).  Then the operator's rows, in boxes of 128, 64 and 32 (the
+      // 128B swizzle is a function of the shared-memory address: they line up as one tile).
+      const CUtensorMap* const mv = &maps.v[it.q];
+      const int m0b = (int)((uint32_t)it.m0 / A2_ROWS);
       for (int e = it.kb; e < it.ke && ok; ++e) {
         const int le = (e - it.kb) & 31;
         if (le == 0 && e > it.kb)
           ent = e + lane < it.ke ? ents[e + lane] : make_int4(0, 0, 0, 0);
         if (e == it.kb && nx.kb + lane < nx.ke) ent_nx = ents[nx.kb + lane];
-        const int f0 = __shfl_sync(0xffffffffu, ent.x, le), f1 = __shfl_sync(0xffffffffu, ent.y, le);
-        const int kdim = __shfl_sync(0xffffffffu, ent.z, le);
+        const int f0 = bcast_uniform(ent.x, le, lane), f1 = bcast_uniform(ent.y, le, lane);
+        const int kdim = bcast_uniform(ent.z, le, lane);
         const int pool = PASS == 0 ? f0 : f1, voff = PASS == 0 ? f1 : f0;
         const int nk = (kdim + BK - 1) / BK;
         for (int kc = 0; kc < nk; ++kc) {
@@ -477,17 +488,26 @@ hv_tc_seg_kernel(const __grid_constant__ GMaps maps, const SParams p) {
           }
           const uint32_t a_s = smem_u32(smem + stage * G_STAGE);
           const uint32_t b_s = a_s + G_STAGE_A;
-          if (lane == 0) mbar_expect_tx(full(stage), tx);
-          __syncwarp();
-          if (bi < 0) {
+          const uint32_t fb = full(stage);
+          if (el) {
+            mbar_expect_tx(fb, tx);
             if (PASS == 0)
-              tma_load_2d(a_s, &maps.vk[it.q], full(stage), voff + kc * BK, it.m0);
+              tma_load_2d(a_s, mv, fb, voff + kc * BK, it.m0);
+            else if (it.a3)
+              tma_load_3d(a_s, mv, fb, 0, voff + kc * BK, m0b);
             else
-              tma_load_2d(a_s + lane * p.a2_lbo, &maps.vm[it.q], full(stage),
-                          it.m0 + lane * p.a2_box_rows, voff + kc * BK);
-          } else if (bi < nb) {
-            tma_load_2d(b_s + bi * 32 * 128, PASS == 0 ? &maps.L : &maps.R, full(stage), kc * BK,
-                        pool + it.n0 + 32 * bi);
+              for (int b = 0; b < G_BM / A2_ROWS; ++b)
+                tma_load_2d(a_s + b * (A2_ROWS * 128), mv, fb, it.m0 + b * A2_ROWS, voff + kc * BK);
+            uint32_t bd = b_s;
+            int br = pool + it.n0;
+            for (int b = nb >> 2; b > 0; --b, bd += 128 * 128, br += 128)
+              tma_load_2d(bd, &maps.op[2], fb, kc * BK, br);
+            if (nb & 2) {
+              tma_load_2d(bd, &maps.op[1], fb, kc * BK, br);
+              bd += 64 * 128;
+              br += 64;
+            }
+            if (nb & 1) tma_load_2d(bd, &maps.op[0], fb, kc * BK, br);
           }
           stage = stage + 1 == G_STAGES ? 0 : stage + 1;
           phase ^= stage == 0 ? 1u : 0u;
@@ -495,6 +515,7 @@ hv_tc_seg_kernel(const __grid_constant__ GMaps maps, const SParams p) {
       }
       if (it.kb == it.ke && nx.kb + lane < nx.ke) ent_nx = ents[nx.kb + lane];
       it = nx;
+      nx = nn;
       ent = ent_nx;
     }
   } else if (warp == 1) {
@@ -503,17 +524,19 @@ hv_tc_seg_kernel(const __grid_constant__ GMaps maps, const SParams p) {
     uint32_t phase = 0;
     int acc = 0;
     uint32_t aphase = 0;
-    const uint64_t a_hi = PASS == 0 ? sdesc(0, 16, 1024) : sdesc(0, p.a2_lbo, p.a2_sbo, p.a2_layout);
-    const uint32_t a_step = PASS == 0 ? 32u : p.a2_kstep;
-    const uint64_t b_hi = sdesc(0, 16, 1024);
-    const int ksteps = BK / p.KSTEP;  // 4
-    const uint32_t el = lane == 0;
+    // operand descriptors of stage 0 (the V tile of pass 2 is MN-major; TF32 in 32-byte atoms)
+    const uint64_t b_hi = sdesc(0, 16, 1024), a_hi = PASS == 0 ? b_hi
+        : sdesc(0, A2_ROWS * 128, BF16 ? 1024 : 512, BF16 ? 2 : 1);
+    constexpr uint32_t A_STEP = PASS == 0 ? 32 : BF16 ? 2048 : 1024;  // bytes per instruction's K
+    const uint64_t a_0 = a_hi | sdesc_addr(smem_u32(smem)),
+                   b_0 = b_hi | sdesc_addr(smem_u32(smem) + G_STAGE_A);
+    const uint32_t el = elect_one();
     bool ok = true;
     int ti = blockIdx.x;
-    SItem it = ti < p.nitems ? p.items[ti] : none;
+    SItem it = item(ti), nx = item(ti + gridDim.x);
     int4 ent = it.kb + lane < it.ke ? ents[it.kb + lane] : make_int4(0, 0, 0, 0);
     for (; ti < p.nitems && ok; ti += gridDim.x) {
-      const SItem nx = ti + (int)gridDim.x < p.nitems ? p.items[ti + gridDim.x] : none;
+      const SItem nn = item(ti + 2 * gridDim.x);
       int4 ent_nx = make_int4(0, 0, 0, 0);
       const int nidx = (min(NMAX, it.sdim - it.n0) + 15) / 16 - 1;
       ok = __all_sync(0xffffffffu, mbar_wait(tempty(acc), aphase ^ 1u, abort));
@@ -529,27 +552,26 @@ hv_tc_seg_kernel(const __grid_constant__ GMaps maps, const SParams p) {
         if (le == 0 && e > it.kb)
           ent = e + lane < it.ke ? ents[e + lane] : make_int4(0, 0, 0, 0);
         if (e == it.kb && nx.kb + lane < nx.ke) ent_nx = ents[nx.kb + lane];
-        const int kdim = __shfl_sync(0xffffffffu, ent.z, le);
-        const int neg = __shfl_sync(0xffffffffu, ent.w, le);
+        const int kdim = bcast_uniform(ent.z, le, lane), neg = bcast_uniform(ent.w, le, lane);
         const uint32_t id = p.idesc[nidx][neg];
         const int nk = (kdim + BK - 1) / BK;
-        const int last = (kdim - (nk - 1) * BK + p.KSTEP - 1) / p.KSTEP;  // steps in the last stage
+        const int last = (kdim - (nk - 1) * BK + KSTEP - 1) / KSTEP;  // steps in the last stage
         for (int kc = 0; kc < nk; ++kc) {
           ok = __all_sync(0xffffffffu, mbar_wait(full(stage), phase, abort));
           if (!ok) {
             if (lane == 0) raise_abort(abort, p.err, 23);
             break;
           }
-          const uint32_t a_s = smem_u32(smem + stage * G_STAGE);
-          const uint32_t b_s = a_s + G_STAGE_A;
-          const int nks = kc + 1 == nk ? last : ksteps;
-#pragma unroll
-          for (int k = 0; k < 4; ++k) {
-            umma_if_t<BF16>(dt, a_hi | sdesc_addr(a_s + k * a_step), b_hi | sdesc_addr(b_s + k * 32),
-                            id, accum, (uint32_t)(k < nks) & el);
-            accum = 1;  // step 0 is always issued
+          const uint64_t a = a_0 + (stage * (G_STAGE >> 4)), b = b_0 + (stage * (G_STAGE >> 4));
+          const int nks = kc + 1 == nk ? last : BK / KSTEP;
+          if (el) {
+            umma_t<BF16>(dt, a, b, id, accum);  // step 0 is always issued
+            if (nks > 1) umma_t<BF16>(dt, a + (A_STEP >> 4), b + 2, id, 1);
+            if (nks > 2) umma_t<BF16>(dt, a + 2 * (A_STEP >> 4), b + 4, id, 1);
+            if (nks > 3) umma_t<BF16>(dt, a + 3 * (A_STEP >> 4), b + 6, id, 1);
+            umma_commit(empty(stage));
           }
-          if (el) umma_commit(empty(stage));
+          accum = 1;
           stage = stage + 1 == G_STAGES ? 0 : stage + 1;
           phase ^= stage == 0 ? 1u : 0u;
         }
@@ -562,6 +584,7 @@ hv_tc_seg_kernel(const __grid_constant__ GMaps maps, const SParams p) {
       }
       if (it.kb == it.ke && nx.kb + lane < nx.ke) ent_nx = ents[nx.kb + lane];
       it = nx;
+      nx = nn;
       ent = ent_nx;
     }
     __syncwarp();
@@ -724,6 +747,36 @@ int map2d(CUtensorMap* m, const void* base, bool bf16, uint64_t inner, uint64_t 
   if (r != CUDA_SUCCESS)
     return set_error(DMRG2D_ECUDA, "cuTensorMapEncodeTiled failed (%d)", (int)r);
   return DMRG2D_OK;
+}
+
+// a matrix of ld x d1 elements as box rows x columns x row blocks of d0: the box's row blocks
+// lie one after another in shared memory, as d2 2-D boxes would
+int map3d(CUtensorMap* m, const void* base, bool bf16, uint64_t d0, uint64_t d1, uint64_t d2,
+          uint64_t ld, uint32_t b0, uint32_t b1, uint32_t b2, CUtensorMapSwizzle swz) {
+  auto fn = encode();
+  if (!fn) return set_error(DMRG2D_ECUDA, "cuTensorMapEncodeTiled unavailable");
+  const uint64_t elt = bf16 ? 2 : 4;
+  cuuint64_t dims[3] = {d0, d1, d2};
+  cuuint64_t strides[2] = {ld * elt, d0 * elt};
+  cuuint32_t box[3] = {b0, b1, b2};
+  cuuint32_t es[3] = {1, 1, 1};
+  CUresult r = fn(m, bf16 ? CU_TENSOR_MAP_DATA_TYPE_BFLOAT16 : CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 3,
+                  const_cast<void*>(base), dims, strides, box, es, CU_TENSOR_MAP_INTERLEAVE_NONE,
+                  swz, CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+  if (r != CUDA_SUCCESS)
+    return set_error(DMRG2D_ECUDA, "cuTensorMapEncodeTiled failed (%d)", (int)r);
+  return DMRG2D_OK;
+}
+
+// Pass 2's V tile as one 3-D box (rows in blocks of 32 or 64): the last block of a column runs
+// on into the next column, whose rows are not stored, and that of V_q's last column into the
+// matrix behind it.  Where that is the end of the vector, 2-D boxes, which stop at ld.
+int seg_one_box(const GroupPlan* g, int q) {
+  long long n = 0;
+  for (int i = 0; i < g->nQ; ++i)
+    n = std::max(n, g->qbase[i] + (long long)g->qld[i] * g->qcols[i]);
+  const long long up = (g->qld[q] + 63) / 64 * 64;
+  return g->qbase[q] + (long long)g->qld[q] * (g->qcols[q] - 1) + up <= n;
 }
 
 template <typename T>
@@ -919,7 +972,7 @@ int gp_finalise(dmrg2d_ops* ops, GroupPlan* g, cudaStream_t s) {
       for (int m0 = 0; m0 < g->qld[q]; m0 += 128)
         for (size_t c = 0; c < g->cols.size(); ++c) {
           if (g->cols[c].q != q) continue;
-          for (int n0 = 0; n0 < g->cols[c].dim; n0 += 256) s2.push_back({q, (int)c, n0, m0, g->cols[c].k2b, g->cols[c].k2e, g->cols[c].dim, 0});
+          for (int n0 = 0; n0 < g->cols[c].dim; n0 += 256) s2.push_back({q, (int)c, n0, m0, g->cols[c].k2b, g->cols[c].k2e, g->cols[c].dim, seg_one_box(g, q)});
         }
     }
     st = gup(D, s1, &D->sitems[0], nb, s);
@@ -978,18 +1031,18 @@ int gp_finalise(dmrg2d_ops* ops, GroupPlan* g, cudaStream_t s) {
       st = map2d(&D->mL[1], D->pL16, true, D->KPL, rowsL, 64, G_BM, CU_TENSOR_MAP_SWIZZLE_128B);
     if (st == DMRG2D_OK)
       st = map2d(&D->mLlo, D->pL16lo, true, D->KPL, rowsL, 64, G_BM, CU_TENSOR_MAP_SWIZZLE_128B);
-    for (int b = 0; b < 2 && st == DMRG2D_OK; ++b) {
-      const bool bf = b == 1;
-      st = map2d(&D->mL32[b], bf ? (const void*)D->pL16 : (const void*)D->pL32, bf, D->KPL,
-                 rowsL, bf ? 64 : 32, 32, CU_TENSOR_MAP_SWIZZLE_128B);
-      if (st == DMRG2D_OK)
-        st = map2d(&D->mR32[b], bf ? (const void*)D->pR16 : (const void*)D->pR32, bf, D->KPR,
-                   rowsR, bf ? 64 : 32, 32, CU_TENSOR_MAP_SWIZZLE_128B);
+    for (int b = 0; b < 3; ++b) {
+      const void* pl[3] = {D->pL32, D->pL16, D->pL16lo};
+      const void* pr[3] = {D->pR32, D->pR16, D->pR16lo};
+      const bool bf = b > 0;
+      for (int i = 0; i < 3 && st == DMRG2D_OK; ++i) {
+        st = map2d(&D->mLs[b][i], pl[b], bf, D->KPL, rowsL, bf ? 64 : 32, 32u << i,
+                   CU_TENSOR_MAP_SWIZZLE_128B);
+        if (st == DMRG2D_OK)
+          st = map2d(&D->mRs[b][i], pr[b], bf, D->KPR, rowsR, bf ? 64 : 32, 32u << i,
+                     CU_TENSOR_MAP_SWIZZLE_128B);
+      }
     }
-    if (st == DMRG2D_OK)
-      st = map2d(&D->mL32lo, D->pL16lo, true, D->KPL, rowsL, 64, 32, CU_TENSOR_MAP_SWIZZLE_128B);
-    if (st == DMRG2D_OK)
-      st = map2d(&D->mR32lo, D->pR16lo, true, D->KPR, rowsR, 64, 32, CU_TENSOR_MAP_SWIZZLE_128B);
     for (int b = 0; b < 2 && st == DMRG2D_OK; ++b) {
       const uint32_t rows_box = b ? 256 : 128;
       st = map2d(&D->mR[0][b], D->pR32, false, D->KPR, rowsR, 32, rows_box,
@@ -1111,16 +1164,24 @@ int gp_launch_seg(const dmrg2d_ops* ops, const GroupPlan* g, const void* v, floa
   const uint32_t BK = bf ? 64 : 32;
   const int elt = bf ? 2 : 4;
   const int box_rows = bf ? 64 : 32;
-  GMaps maps;
-  maps.L = lo_ops ? D->mL32lo : D->mL32[bf ? 1 : 0];  // 32-row boxes of the pools
-  maps.R = lo_ops ? D->mR32lo : D->mR32[bf ? 1 : 0];
+  SMaps maps[2];
+  const int pb = lo_ops ? 2 : bf ? 1 : 0;
+  for (int i = 0; i < 3; ++i) {
+    maps[0].op[i] = D->mLs[pb][i];
+    maps[1].op[i] = D->mRs[pb][i];
+  }
   for (int q = 0; q < g->nQ; ++q) {
     const char* base = (const char*)v + (size_t)g->qbase[q] * elt;
-    D2_TRY(map2d(&maps.vk[q], base, bf, (uint64_t)g->qld[q], (uint64_t)g->qcols[q], BK, 128,
-                 CU_TENSOR_MAP_SWIZZLE_128B));
-    D2_TRY(map2d(&maps.vm[q], base, bf, (uint64_t)g->qld[q], (uint64_t)g->qcols[q],
-                 (uint32_t)box_rows, BK,
-                 bf ? CU_TENSOR_MAP_SWIZZLE_128B : CU_TENSOR_MAP_SWIZZLE_128B_ATOM_32B));
+    const uint64_t ld = (uint64_t)g->qld[q], cols = (uint64_t)g->qcols[q];
+    D2_TRY(map2d(&maps[0].v[q], base, bf, ld, cols, BK, 128, CU_TENSOR_MAP_SWIZZLE_128B));
+    const CUtensorMapSwizzle swz =
+        bf ? CU_TENSOR_MAP_SWIZZLE_128B : CU_TENSOR_MAP_SWIZZLE_128B_ATOM_32B;
+    if (seg_one_box(g, q))
+      D2_TRY(map3d(&maps[1].v[q], base, bf, (uint64_t)box_rows, cols,
+                   (ld + box_rows - 1) / box_rows, ld, (uint32_t)box_rows, BK, G_BM / box_rows,
+                   swz));
+    else
+      D2_TRY(map2d(&maps[1].v[q], base, bf, ld, cols, (uint32_t)box_rows, BK, swz));
   }
   SParams p;
   p.rows = D->rows;
@@ -1132,14 +1193,6 @@ int gp_launch_seg(const dmrg2d_ops* ops, const GroupPlan* g, const void* v, floa
   p.qcols = D->d_qcols;
   p.y = y;
   p.err = D->err;
-  p.a2_box_rows = box_rows;
-  p.a2_boxes = G_BM / box_rows;
-  p.a2_lbo = (uint32_t)box_rows * BK * elt;
-  p.a2_kstep = bf ? 2048 : 1024;
-  p.a2_layout = bf ? 2u : 1u;
-  p.a2_sbo = bf ? 1024u : 512u;
-  p.BK = (int)BK;
-  p.KSTEP = bf ? 16 : 8;
   const int fmt = bf ? 1 : 2;
   auto ev = prof_slot(ops);
   if (ev.first) D2_CUDA(cudaEventRecord(ev.first, s));
@@ -1149,17 +1202,14 @@ int gp_launch_seg(const dmrg2d_ops* ops, const GroupPlan* g, const void* v, floa
     p.accum_y = accum ? 1 : 0;
     for (int i = 0; i < 16; ++i)
       for (int n = 0; n < 2; ++n) p.idesc[i][n] = make_idesc(fmt, pass, G_BM, 16 * (i + 1), 0, n);
-    // A = the V tile (16 KB); B = 32-row boxes of operator rows (4 KB each)
-    p.a_bytes = G_STAGE_A;
-    p.b_box_bytes = 32 * 128;
     if (p.nitems == 0) continue;
     const int grid = std::min(p.nitems, D->sms);
     if (bf) {
-      if (pass) hv_tc_seg_kernel<1, 1><<<grid, G_THREADS, G_SMEM, s>>>(maps, p);
-      else hv_tc_seg_kernel<1, 0><<<grid, G_THREADS, G_SMEM, s>>>(maps, p);
+      if (pass) hv_tc_seg_kernel<1, 1><<<grid, G_THREADS, G_SMEM, s>>>(maps[1], p);
+      else hv_tc_seg_kernel<1, 0><<<grid, G_THREADS, G_SMEM, s>>>(maps[0], p);
     } else {
-      if (pass) hv_tc_seg_kernel<0, 1><<<grid, G_THREADS, G_SMEM, s>>>(maps, p);
-      else hv_tc_seg_kernel<0, 0><<<grid, G_THREADS, G_SMEM, s>>>(maps, p);
+      if (pass) hv_tc_seg_kernel<0, 1><<<grid, G_THREADS, G_SMEM, s>>>(maps[1], p);
+      else hv_tc_seg_kernel<0, 0><<<grid, G_THREADS, G_SMEM, s>>>(maps[0], p);
     }
     D2_CUDA(cudaGetLastError());
   }

@@ -362,9 +362,7 @@ __global__ void __launch_bounds__(FX_THREADS, 1) hv_fx_kernel(const FxParams p) 
     if (warp == FX_CONV) {
       uint32_t st = 0, g = 0, next = 0, first = 0;  // g: current group
       bool ok = true;
-      uint32_t el;
-      asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.u32 %0, 1, 0, p;\n\t}"
-                   : "=r"(el));
+      const uint32_t el = elect_one();
       // V: pass 0 K-major (K cores 2048 apart, row cores 128), pass 1 MN-major
       const uint64_t ah = PASS == 0 ? sdesc(0, FX_LONG * 16, 128, 0) : sdesc(0, 128, FX_K * 16, 0);
       const uint64_t bh = sdesc(0, 128, FX_K * 16, 0);
