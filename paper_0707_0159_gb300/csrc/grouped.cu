@@ -113,7 +113,7 @@ hv_tc_grouped_kernel(const __grid_constant__ GMaps maps, const GParams p) {
   uint64_t* bars = (uint64_t*)(smem + G_STAGES * G_STAGE);
   uint32_t* tmem_slot = (uint32_t*)(bars + 2 * G_STAGES + 4);
   volatile int* abort = (volatile int*)(tmem_slot + 1);
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = warp_index(), lane = threadIdx.x & 31;
   auto full = [&](int s) { return smem_u32(bars + s); };
   auto empty = [&](int s) { return smem_u32(bars + G_STAGES + s); };
   auto tfull = [&](int b) { return smem_u32(bars + 2 * G_STAGES + b); };
@@ -145,11 +145,12 @@ hv_tc_grouped_kernel(const __grid_constant__ GMaps maps, const GParams p) {
   const uint32_t tmem_base = *tmem_slot;
   const int BK = p.BK;
 
-  if (warp == 0 && lane == 0) {
+  if (warp == 0) {
     // ------------------------------- TMA producer -------------------------------
+    const uint32_t el = elect_one();
     int stage = 0;
     uint32_t phase = 0;
-    for (int ti = blockIdx.x; ti < p.ntiles && !*abort; ti += gridDim.x) {
+    for (int ti = blockIdx.x; ti < p.ntiles; ti += gridDim.x) {
       const GTile t = p.tiles[ti];
       const GRow rs = p.rows[t.rs];
       const GCol cs = p.cols[t.cs];
@@ -173,21 +174,23 @@ hv_tc_grouped_kernel(const __grid_constant__ GMaps maps, const GParams p) {
           }
           const int nk = (kdim + BK - 1) / BK;
           for (int kc = 0; kc < nk; ++kc) {
-            if (!mbar_wait(empty(stage), phase ^ 1u, abort)) {
-              raise_abort(abort, p.err, 11);
+            if (!__all_sync(0xffffffffu, mbar_wait(empty(stage), phase ^ 1u, abort))) {
+              if (el) raise_abort(abort, p.err, 11);
               goto producer_done;
             }
             const uint32_t a_s = smem_u32(smem + stage * G_STAGE);
             const uint32_t b_s = a_s + G_STAGE_A;
-            mbar_expect_tx(full(stage), p.tx_bytes);
-            if (ph == 0) {
-              tma_load_2d(a_s, &maps.L, full(stage), kc * BK, a_pool + t.r_in);
-              tma_load_2d(b_s, vk, full(stage), b_row + kc * BK, c0);
-            } else {
-              for (int b = 0; b < p.a2_boxes; ++b)
-                tma_load_2d(a_s + b * p.a2_lbo, vm, full(stage), r0 + b * p.a2_box_rows,
-                            a_col + kc * BK);
-              tma_load_2d(b_s, &maps.R, full(stage), kc * BK, b_pool + t.c_in);
+            if (el) {
+              mbar_expect_tx(full(stage), p.tx_bytes);
+              if (ph == 0) {
+                tma_load_2d(a_s, &maps.L, full(stage), kc * BK, a_pool + t.r_in);
+                tma_load_2d(b_s, vk, full(stage), b_row + kc * BK, c0);
+              } else {
+                for (int b = 0; b < p.a2_boxes; ++b)
+                  tma_load_2d(a_s + b * p.a2_lbo, vm, full(stage), r0 + b * p.a2_box_rows,
+                              a_col + kc * BK);
+                tma_load_2d(b_s, &maps.R, full(stage), kc * BK, b_pool + t.c_in);
+              }
             }
             if (++stage == G_STAGES) {
               stage = 0;
@@ -197,19 +200,21 @@ hv_tc_grouped_kernel(const __grid_constant__ GMaps maps, const GParams p) {
         }
       }
     }
-  producer_done:;
-  } else if (warp == 1 && lane == 0) {
+  producer_done:
+    __syncwarp();
+  } else if (warp == 1) {
     // ------------------------------- MMA issuer ---------------------------------
+    const uint32_t el = elect_one();
     int stage = 0;
     uint32_t phase = 0;
     int acc = 0;
     uint32_t aphase = 0;
-    for (int ti = blockIdx.x; ti < p.ntiles && !*abort; ti += gridDim.x) {
+    for (int ti = blockIdx.x; ti < p.ntiles; ti += gridDim.x) {
       const GTile t = p.tiles[ti];
       const GRow rs = p.rows[t.rs];
       const GCol cs = p.cols[t.cs];
-      if (!mbar_wait(tempty(acc), aphase ^ 1u, abort)) {
-        raise_abort(abort, p.err, 12);
+      if (!__all_sync(0xffffffffu, mbar_wait(tempty(acc), aphase ^ 1u, abort))) {
+        if (el) raise_abort(abort, p.err, 12);
         break;
       }
       tc_fence_after();
@@ -220,10 +225,11 @@ hv_tc_grouped_kernel(const __grid_constant__ GMaps maps, const GParams p) {
         const int e0 = ph == 0 ? rs.k1b : cs.k2b, e1 = ph == 0 ? rs.k1e : cs.k2e;
         // descriptor fields fixed for the phase (no branch between two MMAs: the tensor
         // pipe's instruction queue is shallow)
-        const uint64_t a_hi = ph == 0 ? sdesc(0, 16, 1024)
-                                      : sdesc(0, p.a2_lbo, p.a2_sbo, p.a2_layout);
-        const uint32_t a_step = ph == 0 ? 32u : p.a2_kstep;
-        const uint64_t b_hi = sdesc(0, 16, 1024);
+        const uint64_t a_0 = sdesc_addr(smem_u32(smem)) |
+                             (ph == 0 ? sdesc(0, 16, 1024)
+                                      : sdesc(0, p.a2_lbo, p.a2_sbo, p.a2_layout));
+        const uint32_t a_step = (ph == 0 ? 32u : p.a2_kstep) >> 4;
+        const uint64_t b_0 = sdesc_addr(smem_u32(smem) + G_STAGE_A) | sdesc(0, 16, 1024);
         for (int e = e0; e < e1 && ok; ++e) {
           const int kdim = ph == 0 ? p.k1[e].kdim : p.k2[e].kdim;
           const int neg = ph == 0 ? p.k1[e].neg : p.k2[e].neg;
@@ -232,32 +238,33 @@ hv_tc_grouped_kernel(const __grid_constant__ GMaps maps, const GParams p) {
           const int nk = (kdim + BK - 1) / BK;
           for (int kc = 0; kc < nk; ++kc) {
             // the mbarrier's completion orders the TMA writes before these MMAs
-            if (!mbar_wait(full(stage), phase, abort)) {
-              raise_abort(abort, p.err, 13);
+            if (!__all_sync(0xffffffffu, mbar_wait(full(stage), phase, abort))) {
+              if (el) raise_abort(abort, p.err, 13);
               ok = false;
               break;
             }
-            const uint32_t a_s = smem_u32(smem + stage * G_STAGE);
-            const uint32_t b_s = a_s + G_STAGE_A;
-#pragma unroll
-            for (int k = 0; k < 4; ++k) {
-              umma_t<BF16>(dt, a_hi | sdesc_addr(a_s + k * a_step),
-                           b_hi | sdesc_addr(b_s + k * 32), id, accum);
-              accum = 1;
+            const uint64_t a = a_0 + stage * (G_STAGE >> 4), b = b_0 + stage * (G_STAGE >> 4);
+            if (el) {
+              umma_t<BF16>(dt, a, b, id, accum);
+              umma_t<BF16>(dt, a + a_step, b + 2, id, 1);
+              umma_t<BF16>(dt, a + 2 * a_step, b + 4, id, 1);
+              umma_t<BF16>(dt, a + 3 * a_step, b + 6, id, 1);
+              umma_commit(empty(stage));
             }
-            umma_commit(empty(stage));
+            accum = 1;
             stage = stage + 1 == G_STAGES ? 0 : stage + 1;
             phase ^= stage == 0 ? 1u : 0u;
           }
         }
       }
       if (!ok) break;
-      umma_commit(tfull(acc));
+      if (el) umma_commit(tfull(acc));
       if (++acc == 2) {
         acc = 0;
         aphase ^= 1u;
       }
     }
+    __syncwarp();
   } else if (warp >= 2) {
     // ------------------------------- epilogue -----------------------------------
     // two warps per TMEM lane quadrant, alternating 32-column chunks; the scalar moves of

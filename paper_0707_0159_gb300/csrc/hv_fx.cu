@@ -23,11 +23,12 @@
 // What bounds it: the digit arithmetic, about 25 instructions per entry of the two operands,
 // most of them on the half-rate integer pipe (3600-4800 cycles a stage of 128 x 64 x 32, at
 // 45 % of the integer pipe: three warps on an SM quarter do not hide its latencies), and the
-// addition of the diagonals (5000-8000 cycles a group, during which no MMA runs); the MMAs
-// themselves are 1800 cycles a stage.  Measured against float pairs on the FP32 pipes (12
+// addition of the diagonals (5000-8000 cycles a group, during which no MMA runs).  The MMAs
+// took 1800 cycles a stage with a guard predicate on each (84 to issue one); issued in a block
+// of one elected lane they take half (dense m = 128 10.40 -> 9.65 ms).  Measured against float pairs on the FP32 pipes (12
 // FP32 operations per product, pieces of 64 x 64):
-//   3-leg Hubbard dense, m = 128          73.6 -> 10.3 ms (23 TFLOP/s), error 1.7e-13 -> 3.3e-14
-//   4-leg Heisenberg sectors, m = 512     16.8 -> 2.06 ms,              error 2.6e-13 -> 1.5e-14
+//   3-leg Hubbard dense, m = 128          73.6 -> 9.65 ms (25 TFLOP/s), error 1.7e-13 -> 3.3e-14
+//   4-leg Heisenberg sectors, m = 512     16.8 -> 1.89 ms,              error 2.6e-13 -> 1.5e-14
 //   3-leg Hubbard sectors, m = 256        44.7 -> 1.78 ms
 // Tried and left out: 8 instead of 12 conversion warps, one warp role for conversion and
 // addition (17 ms), the swizzled operand layouts (11.0 ms), one accumulation per stage
@@ -181,7 +182,7 @@ __global__ void __launch_bounds__(FX_THREADS, 1) hv_fx_kernel(const FxParams p) 
   volatile int* abort = (volatile int*)(tmem_slot + 1);
   // accumulation group g: ginfo[g % 4] = 2 * first stage + (last group of its item)
   volatile uint32_t* ginfo = (volatile uint32_t*)(tmem_slot + 2);
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = warp_index(), lane = threadIdx.x & 31;
   auto ready = [&](int b) { return smem_u32(bars + b); };
   auto freeb = [&](int b) { return smem_u32(bars + 2 + b); };
   const uint32_t tfull = smem_u32(bars + 4), tempty = smem_u32(bars + 5);
@@ -407,19 +408,19 @@ __global__ void __launch_bounds__(FX_THREADS, 1) hv_fx_kernel(const FxParams p) 
           const uint64_t a0 = ah | sdesc_addr(sa), b0 = bh | sdesc_addr(sa + FX_S * FX_A);
           uint32_t n;  // opaque: keeps the instruction descriptors out of the outer loops
           asm volatile("mov.u32 %0, %1;" : "=r"(n) : "r"(N));
-#pragma unroll
-          for (int k = 0; k < 2; ++k)
-#pragma unroll
-            for (int i = 0; i < FX_S; ++i) {
-              const uint32_t w = n * (FX_S - i);  // columns of diagonals i .. 6
-              const uint64_t a = a0 + ((i * FX_A + k * AK) >> 4), bb = b0 + ((k * 256) >> 4);
-              const uint32_t dt = tmem + n * i, acc = k > 0 || i > 0 || !fresh;
-              umma_if_t<1>(dt, a, bb, id | (min(w, 256u) >> 3) << 17, acc, el);
-              if (i < 3)  // N = 48 or 64: the columns above 256
-                umma_if_t<1>(dt + 256, a, bb + ((256 / 8 * FX_K * 16) >> 4),
-                             id | ((w - 256) >> 3) << 17, acc, w > 256 ? el : 0);
-            }
           if (el) {
+#pragma unroll
+            for (int k = 0; k < 2; ++k)
+#pragma unroll
+              for (int i = 0; i < FX_S; ++i) {
+                const uint32_t w = n * (FX_S - i);  // columns of diagonals i .. 6
+                const uint64_t a = a0 + ((i * FX_A + k * AK) >> 4), bb = b0 + ((k * 256) >> 4);
+                const uint32_t dt = tmem + n * i, acc = k > 0 || i > 0 || !fresh;
+                umma_t<1>(dt, a, bb, id | (min(w, 256u) >> 3) << 17, acc);
+                if (i < 3 && w > 256)  // N = 48 or 64: the columns above 256
+                  umma_t<1>(dt + 256, a, bb + ((256 / 8 * FX_K * 16) >> 4),
+                            id | ((w - 256) >> 3) << 17, acc);
+              }
             umma_commit(freeb(b));
             if (last) umma_commit(tfull);
           }

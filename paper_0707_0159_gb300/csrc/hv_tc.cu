@@ -170,7 +170,7 @@ hv_tc_kernel(const __grid_constant__ CUtensorMap mHL, const __grid_constant__ CU
   uint64_t* bars = (uint64_t*)(smem + STAGES * STAGE_BYTES);
   uint32_t* tmem_slot = (uint32_t*)(bars + 2 * STAGES + 4);
   volatile int* abort = (volatile int*)(tmem_slot + 1);
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = warp_index(), lane = threadIdx.x & 31;
   auto full = [&](int s) { return smem_u32(bars + s); };
   auto empty = [&](int s) { return smem_u32(bars + STAGES + s); };
   auto tfull = [&](int b) { return smem_u32(bars + 2 * STAGES + b); };
@@ -201,45 +201,46 @@ hv_tc_kernel(const __grid_constant__ CUtensorMap mHL, const __grid_constant__ CU
   tc_fence_after();
   const uint32_t tmem_base = *tmem_slot;
 
-  if (warp == 0 && lane == 0) {
+  if (warp == 0) {
     // ------------------------------- TMA producer -------------------------------
+    const uint32_t el = elect_one();
     int stage = 0;
     uint32_t phase = 0;
-    for (int t = blockIdx.x; t < p.tiles && !*abort; t += gridDim.x) {
+    const int repL = (int)(blockIdx.x % p.copies) * p.poolL_rows;  // this CTA's pool replica
+    const int repR = (int)(blockIdx.x % p.copies) * p.poolR_rows;
+    for (int t = blockIdx.x; t < p.tiles; t += gridDim.x) {
       const TileCoord c = decode(p, t);
       const int r0 = c.i2 * p.m1 + c.mt * BM;
-      const int c0 = c.i3 * p.m4 + c.nt * p.BN;
+      const int c0 = c.i3 * p.m4 + c.nt * p.BN, r0b = r0 / p.a2_box_rows;
       for (int ph = p.ph0; ph < p.ph1; ++ph) {
         const int e0 = ph == 0 ? p.Lptr[c.i2] : p.Rptr[c.i3];
         const int e1 = ph == 0 ? p.Lptr[c.i2 + 1] : p.Rptr[c.i3 + 1];
         const int kb = ph == 0 ? p.kblk1 : p.kblk2;
         for (int e = e0; e < e1; ++e) {
           const int nb = ph == 0 ? p.Lcol[e] : p.Rcol[e];
+          const int op_row = ph == 0 ? (p.pooled ? p.k1[e].a_pool + repL : e * p.m1) + c.mt * BM
+                                     : (p.pooled ? p.k2[e].b_pool + repR : e * p.m4) + c.nt * p.BN;
           for (int kc = 0; kc < kb; ++kc) {
-            if (!mbar_wait(empty(stage), phase ^ 1u, abort)) {
-              raise_abort(abort, p.err, 1);
+            if (!__all_sync(0xffffffffu, mbar_wait(empty(stage), phase ^ 1u, abort))) {
+              if (el) raise_abort(abort, p.err, 1);
               goto producer_done;
             }
             const uint32_t a_s = smem_u32(smem + stage * STAGE_BYTES);
             const uint32_t b_s = a_s + STAGE_A;
-            mbar_expect_tx(full(stage), p.tx_bytes);
-            if (ph == 0) {
-              tma_load_2d(a_s, &mHL, full(stage), kc * p.BK,
-                          (p.pooled ? p.k1[e].a_pool + (int)(blockIdx.x % p.copies) * p.poolL_rows
-                                    : e * p.m1) +
-                              c.mt * BM);
-              tma_load_2d(b_s, &mVk, full(stage), nb * p.m1 + kc * p.BK, c0);
-            } else {
-              if (p.a2_3d)
-                tma_load_3d(a_s, &mVm, full(stage), 0, nb * p.m4 + kc * p.BK, r0 / p.a2_box_rows);
-              else
-                for (int b = 0; b < p.a2_boxes; ++b)
-                  tma_load_2d(a_s + b * p.a2_lbo, &mVm, full(stage), r0 + b * p.a2_box_rows,
-                              nb * p.m4 + kc * p.BK);
-              tma_load_2d(b_s, &mHR, full(stage), kc * p.BK,
-                          (p.pooled ? p.k2[e].b_pool + (int)(blockIdx.x % p.copies) * p.poolR_rows
-                                    : e * p.m4) +
-                              c.nt * p.BN);
+            if (el) {
+              mbar_expect_tx(full(stage), p.tx_bytes);
+              if (ph == 0) {
+                tma_load_2d(a_s, &mHL, full(stage), kc * p.BK, op_row);
+                tma_load_2d(b_s, &mVk, full(stage), nb * p.m1 + kc * p.BK, c0);
+              } else {
+                if (p.a2_3d)
+                  tma_load_3d(a_s, &mVm, full(stage), 0, nb * p.m4 + kc * p.BK, r0b);
+                else
+                  for (int b = 0; b < p.a2_boxes; ++b)
+                    tma_load_2d(a_s + b * p.a2_lbo, &mVm, full(stage), r0 + b * p.a2_box_rows,
+                                nb * p.m4 + kc * p.BK);
+                tma_load_2d(b_s, &mHR, full(stage), kc * p.BK, op_row);
+              }
             }
             if (++stage == STAGES) {
               stage = 0;
@@ -249,17 +250,19 @@ hv_tc_kernel(const __grid_constant__ CUtensorMap mHL, const __grid_constant__ CU
         }
       }
     }
-  producer_done:;
-  } else if (warp == 1 && lane == 0) {
+  producer_done:
+    __syncwarp();
+  } else if (warp == 1) {
     // ------------------------------- MMA issuer ---------------------------------
+    const uint32_t el = elect_one();
     int stage = 0;
     uint32_t phase = 0;
     int acc = 0;
     uint32_t aphase = 0;
-    for (int t = blockIdx.x; t < p.tiles && !*abort; t += gridDim.x) {
+    for (int t = blockIdx.x; t < p.tiles; t += gridDim.x) {
       const TileCoord c = decode(p, t);
-      if (!mbar_wait(tempty(acc), aphase ^ 1u, abort)) {
-        raise_abort(abort, p.err, 2);
+      if (!__all_sync(0xffffffffu, mbar_wait(tempty(acc), aphase ^ 1u, abort))) {
+        if (el) raise_abort(abort, p.err, 2);
         break;
       }
       tc_fence_after();
@@ -271,10 +274,11 @@ hv_tc_kernel(const __grid_constant__ CUtensorMap mHL, const __grid_constant__ CU
         const int e1 = ph == 0 ? p.Lptr[c.i2 + 1] : p.Rptr[c.i3 + 1];
         const int kb = ph == 0 ? p.kblk1 : p.kblk2;
         // descriptor fields fixed for the phase (the A operand of phase 2 is V, MN-major)
-        const uint64_t a_hi = ph == 0 ? sdesc(0, 16, 1024)
-                                      : sdesc(0, p.a2_lbo, p.a2_sbo, p.a2_layout);
-        const uint32_t a_step = ph == 0 ? 32u : p.a2_kstep;
-        const uint64_t b_hi = sdesc(0, 16, 1024);
+        const uint64_t a_0 = sdesc_addr(smem_u32(smem)) |
+                             (ph == 0 ? sdesc(0, 16, 1024)
+                                      : sdesc(0, p.a2_lbo, p.a2_sbo, p.a2_layout));
+        const uint32_t a_step = (ph == 0 ? 32u : p.a2_kstep) >> 4;
+        const uint64_t b_0 = sdesc_addr(smem_u32(smem) + STAGE_A) | sdesc(0, 16, 1024);
         for (int e = e0; e < e1 && ok; ++e) {
           // instruction descriptor of this operator block, chosen once per block
           const int neg = p.pooled ? (ph == 0 ? p.k1[e].neg : p.k2[e].neg) : 0;
@@ -283,32 +287,33 @@ hv_tc_kernel(const __grid_constant__ CUtensorMap mHL, const __grid_constant__ CU
           for (int kc = 0; kc < kb; ++kc) {
             // the mbarrier's completion orders the TMA writes before these MMAs; no
             // tcgen05 fence is needed per stage
-            if (!mbar_wait(full(stage), phase, abort)) {
-              raise_abort(abort, p.err, 3);
+            if (!__all_sync(0xffffffffu, mbar_wait(full(stage), phase, abort))) {
+              if (el) raise_abort(abort, p.err, 3);
               ok = false;
               break;
             }
-            const uint32_t a_s = smem_u32(smem + stage * STAGE_BYTES);
-            const uint32_t b_s = a_s + STAGE_A;
-#pragma unroll
-            for (int k = 0; k < 4; ++k) {
-              umma_t<BF16>(dt, a_hi | sdesc_addr(a_s + k * a_step),
-                           b_hi | sdesc_addr(b_s + k * 32), idb, accum);
-              accum = 1;
+            const uint64_t a = a_0 + stage * (STAGE_BYTES >> 4), b = b_0 + stage * (STAGE_BYTES >> 4);
+            if (el) {
+              umma_t<BF16>(dt, a, b, idb, accum);
+              umma_t<BF16>(dt, a + a_step, b + 2, idb, 1);
+              umma_t<BF16>(dt, a + 2 * a_step, b + 4, idb, 1);
+              umma_t<BF16>(dt, a + 3 * a_step, b + 6, idb, 1);
+              umma_commit(empty(stage));
             }
-            umma_commit(empty(stage));
+            accum = 1;
             stage = stage + 1 == STAGES ? 0 : stage + 1;
             phase ^= stage == 0 ? 1u : 0u;
           }
         }
       }
       if (!ok) break;
-      umma_commit(tfull(acc));
+      if (el) umma_commit(tfull(acc));
       if (++acc == 2) {
         acc = 0;
         aphase ^= 1u;
       }
     }
+    __syncwarp();
   } else if (warp >= 2) {
     // ------------------------------- epilogue -----------------------------------
     const int q = warp & 3;             // TMEM lane quadrant this warp may access
@@ -373,7 +378,7 @@ hv_tc_pair_kernel(const __grid_constant__ CUtensorMap mHL, const __grid_constant
   uint64_t* bars = (uint64_t*)(smem + P_STAGES * P_STAGE);
   uint32_t* tmem_slot = (uint32_t*)(bars + 2 * P_STAGES + 4);
   volatile int* abort = (volatile int*)(tmem_slot + 1);
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = warp_index(), lane = threadIdx.x & 31;
   const uint32_t rank = cluster_ctarank();
   const bool even = rank == 0;
   auto full = [&](int s) { return smem_u32(bars + s); };
@@ -408,14 +413,17 @@ hv_tc_pair_kernel(const __grid_constant__ CUtensorMap mHL, const __grid_constant
   const uint32_t tmem_base = *tmem_slot;
   const int cid = (int)cluster_id_x(), ncl = (int)ncluster_x();
 
-  if (warp == 0 && lane == 0) {
+  if (warp == 0) {
     // ------------------------- TMA producer (both CTAs) -------------------------
+    const uint32_t el = elect_one();
     int stage = 0;
     uint32_t phase = 0;
-    for (int t = cid; t < p.tiles && !*abort; t += ncl) {
+    const int repL = (int)(cid % p.copies) * p.poolL_rows;  // this pair's pool replica
+    const int repR = (int)(cid % p.copies) * p.poolR_rows;
+    for (int t = cid; t < p.tiles; t += ncl) {
       const TileCoord c = decode(p, t);  // c.mt: pair of 128-row pieces
       const int mt = 2 * c.mt + (int)rank;
-      const int r0 = c.i2 * p.m1 + mt * BM;
+      const int r0 = c.i2 * p.m1 + mt * BM, r0b = r0 / p.a2_box_rows;
       const int cb = c.nt * p.BN + (int)rank * P_HALF;  // this CTA's B columns
       for (int ph = p.ph0; ph < p.ph1; ++ph) {
         const int e0 = ph == 0 ? p.Lptr[c.i2] : p.Rptr[c.i3];
@@ -423,30 +431,30 @@ hv_tc_pair_kernel(const __grid_constant__ CUtensorMap mHL, const __grid_constant
         const int kb = ph == 0 ? p.kblk1 : p.kblk2;
         for (int e = e0; e < e1; ++e) {
           const int nb = ph == 0 ? p.Lcol[e] : p.Rcol[e];
+          const int op_row = ph == 0 ? (p.pooled ? p.k1[e].a_pool + repL : e * p.m1) + mt * BM
+                                     : (p.pooled ? p.k2[e].b_pool + repR : e * p.m4) + cb;
           for (int kc = 0; kc < kb; ++kc) {
-            if (!mbar_wait(empty(stage), phase ^ 1u, abort)) {
-              raise_abort(abort, p.err, 11);
+            if (!__all_sync(0xffffffffu, mbar_wait(empty(stage), phase ^ 1u, abort))) {
+              if (el) raise_abort(abort, p.err, 11);
               goto producer_done;
             }
             const uint32_t a_s = smem_u32(smem + stage * P_STAGE);
             const uint32_t b_s = a_s + P_STAGE_A;
-            if (even) mbar_expect_tx(full(stage), 2 * p.tx_bytes);
-            const uint32_t fb = mapa(full(stage), 0);
-            if (ph == 0) {
-              const int arow = p.pooled ? p.k1[e].a_pool + (int)(cid % p.copies) * p.poolL_rows
-                                        : e * p.m1;
-              tma_load_2d_pair(a_s, &mHL, fb, kc * p.BK, arow + mt * BM);
-              tma_load_2d_pair(b_s, &mVk, fb, nb * p.m1 + kc * p.BK, c.i3 * p.m4 + cb);
-            } else {
-              if (p.a2_3d)
-                tma_load_3d_pair(a_s, &mVm, fb, 0, nb * p.m4 + kc * p.BK, r0 / p.a2_box_rows);
-              else
-                for (int b = 0; b < p.a2_boxes; ++b)
-                  tma_load_2d_pair(a_s + b * p.a2_lbo, &mVm, fb, r0 + b * p.a2_box_rows,
-                                   nb * p.m4 + kc * p.BK);
-              const int brow = p.pooled ? p.k2[e].b_pool + (int)(cid % p.copies) * p.poolR_rows
-                                        : e * p.m4;
-              tma_load_2d_pair(b_s, &mHR, fb, kc * p.BK, brow + cb);
+            if (el) {
+              if (even) mbar_expect_tx(full(stage), 2 * p.tx_bytes);
+              const uint32_t fb = mapa(full(stage), 0);
+              if (ph == 0) {
+                tma_load_2d_pair(a_s, &mHL, fb, kc * p.BK, op_row);
+                tma_load_2d_pair(b_s, &mVk, fb, nb * p.m1 + kc * p.BK, c.i3 * p.m4 + cb);
+              } else {
+                if (p.a2_3d)
+                  tma_load_3d_pair(a_s, &mVm, fb, 0, nb * p.m4 + kc * p.BK, r0b);
+                else
+                  for (int b = 0; b < p.a2_boxes; ++b)
+                    tma_load_2d_pair(a_s + b * p.a2_lbo, &mVm, fb, r0 + b * p.a2_box_rows,
+                                     nb * p.m4 + kc * p.BK);
+                tma_load_2d_pair(b_s, &mHR, fb, kc * p.BK, op_row);
+              }
             }
             if (++stage == P_STAGES) {
               stage = 0;
@@ -456,17 +464,19 @@ hv_tc_pair_kernel(const __grid_constant__ CUtensorMap mHL, const __grid_constant
         }
       }
     }
-  producer_done:;
-  } else if (warp == 1 && lane == 0 && even) {
+  producer_done:
+    __syncwarp();
+  } else if (warp == 1 && even) {
     // ------------------------- MMA issuer (even CTA) ----------------------------
+    const uint32_t el = elect_one();
     int stage = 0;
     uint32_t phase = 0;
     int acc = 0;
     uint32_t aphase = 0;
-    for (int t = cid; t < p.tiles && !*abort; t += ncl) {
+    for (int t = cid; t < p.tiles; t += ncl) {
       const TileCoord c = decode(p, t);
-      if (!mbar_wait(tempty(acc), aphase ^ 1u, abort)) {
-        raise_abort(abort, p.err, 12);
+      if (!__all_sync(0xffffffffu, mbar_wait(tempty(acc), aphase ^ 1u, abort))) {
+        if (el) raise_abort(abort, p.err, 12);
         break;
       }
       tc_fence_after();
@@ -478,10 +488,11 @@ hv_tc_pair_kernel(const __grid_constant__ CUtensorMap mHL, const __grid_constant
         const int e1 = ph == 0 ? p.Lptr[c.i2 + 1] : p.Rptr[c.i3 + 1];
         const int kb = ph == 0 ? p.kblk1 : p.kblk2;
         // descriptor fields fixed for the phase (the A operand of phase 2 is V, MN-major)
-        const uint64_t a_hi = ph == 0 ? sdesc(0, 16, 1024)
-                                      : sdesc(0, p.a2_lbo, p.a2_sbo, p.a2_layout);
-        const uint32_t a_step = ph == 0 ? 32u : p.a2_kstep;
-        const uint64_t b_hi = sdesc(0, 16, 1024);
+        const uint64_t a_0 = sdesc_addr(smem_u32(smem)) |
+                             (ph == 0 ? sdesc(0, 16, 1024)
+                                      : sdesc(0, p.a2_lbo, p.a2_sbo, p.a2_layout));
+        const uint32_t a_step = (ph == 0 ? 32u : p.a2_kstep) >> 4;
+        const uint64_t b_0 = sdesc_addr(smem_u32(smem) + P_STAGE_A) | sdesc(0, 16, 1024);
         for (int e = e0; e < e1 && ok; ++e) {
           // instruction descriptor of this operator block, chosen once per block
           const int neg = p.pooled ? (ph == 0 ? p.k1[e].neg : p.k2[e].neg) : 0;
@@ -490,32 +501,33 @@ hv_tc_pair_kernel(const __grid_constant__ CUtensorMap mHL, const __grid_constant
           for (int kc = 0; kc < kb; ++kc) {
             // the mbarrier's completion orders the TMA writes before these MMAs; no
             // tcgen05 fence is needed per stage
-            if (!mbar_wait(full(stage), phase, abort)) {
-              raise_abort(abort, p.err, 13);
+            if (!__all_sync(0xffffffffu, mbar_wait(full(stage), phase, abort))) {
+              if (el) raise_abort(abort, p.err, 13);
               ok = false;
               break;
             }
-            const uint32_t a_s = smem_u32(smem + stage * P_STAGE);
-            const uint32_t b_s = a_s + P_STAGE_A;
-#pragma unroll
-            for (int k = 0; k < 4; ++k) {
-              umma_pair_t<BF16>(dt, a_hi | sdesc_addr(a_s + k * a_step),
-                                b_hi | sdesc_addr(b_s + k * 32), idb, accum);
-              accum = 1;
+            const uint64_t a = a_0 + stage * (P_STAGE >> 4), b = b_0 + stage * (P_STAGE >> 4);
+            if (el) {
+              umma_pair_t<BF16>(dt, a, b, idb, accum);
+              umma_pair_t<BF16>(dt, a + a_step, b + 2, idb, 1);
+              umma_pair_t<BF16>(dt, a + 2 * a_step, b + 4, idb, 1);
+              umma_pair_t<BF16>(dt, a + 3 * a_step, b + 6, idb, 1);
+              umma_commit_pair(empty(stage));
             }
-            umma_commit_pair(empty(stage));
+            accum = 1;
             stage = stage + 1 == P_STAGES ? 0 : stage + 1;
             phase ^= stage == 0 ? 1u : 0u;
           }
         }
       }
       if (!ok) break;
-      umma_commit_pair(tfull(acc));
+      if (el) umma_commit_pair(tfull(acc));
       if (++acc == 2) {
         acc = 0;
         aphase ^= 1u;
       }
     }
+    __syncwarp();
   } else if (warp >= 2) {
     // ------------------------- epilogue (both CTAs) -----------------------------
     const int q = warp & 3;

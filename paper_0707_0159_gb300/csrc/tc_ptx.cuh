@@ -81,7 +81,10 @@ __device__ __forceinline__ uint64_t sdesc(uint32_t addr, uint32_t lbo, uint32_t 
 // `if (elected)` blocks.  These instructions take their operands from uniform registers; where
 // the compiler can see that warp index, loop state and addresses are the warp's own, they are
 // computed there, otherwise each operand is moved over, one instruction after another.  Cycles
-// an instruction, segment kernel, TF32: MMA 84 -> 42, TMA 110 .. 125 -> 45.
+// an instruction, segment kernel, TF32: MMA 84 -> 42, TMA 110 .. 125 -> 45 (a guard predicate on
+// each MMA, without the block: 84).  H·v: dense TF32 3-leg Heisenberg m = 256 43.1 -> 37.2 us,
+// BF16 m = 512 117.9 -> 101.9 us, 2-leg Hubbard m = 384 TF32 525 -> 484 us; FP64X 3-leg Hubbard
+// m = 128 10.40 -> 9.65 ms.
 
 // the warp's index, through a shuffle: uniform for the compiler, so the roles' branches are
 __device__ __forceinline__ int warp_index() {
@@ -191,22 +194,6 @@ __device__ __forceinline__ void umma_t(uint32_t dt, uint64_t a, uint64_t b, uint
         "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
         "tcgen05.mma.cta_group::1.kind::tf32 [%0], %1, %2, %3, p;\n\t}" ::"r"(dt),
         "l"(a), "l"(b), "r"(idesc), "r"(acc));
-}
-// the same, issued only when `go` is nonzero (a guard predicate inside the instruction
-// block: no branch in the issuing thread)
-template <int BF16>
-__device__ __forceinline__ void umma_if_t(uint32_t dt, uint64_t a, uint64_t b, uint32_t idesc,
-                                          uint32_t acc, uint32_t go) {
-  if constexpr (BF16)
-    asm volatile(
-        "{\n\t.reg .pred p, g;\n\tsetp.ne.b32 p, %4, 0;\n\tsetp.ne.b32 g, %5, 0;\n\t"
-        "@g tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(dt),
-        "l"(a), "l"(b), "r"(idesc), "r"(acc), "r"(go));
-  else
-    asm volatile(
-        "{\n\t.reg .pred p, g;\n\tsetp.ne.b32 p, %4, 0;\n\tsetp.ne.b32 g, %5, 0;\n\t"
-        "@g tcgen05.mma.cta_group::1.kind::tf32 [%0], %1, %2, %3, p;\n\t}" ::"r"(dt),
-        "l"(a), "l"(b), "r"(idesc), "r"(acc), "r"(go));
 }
 template <int BF16>
 __device__ __forceinline__ void umma_pair_t(uint32_t dt, uint64_t a, uint64_t b, uint32_t idesc,
