@@ -813,7 +813,7 @@ def lanczos_latency(ops, n, dev, steps=200):
 def time_to_energy(ops, n, prec, args, dev):
     """Ground energy to a residual of tol*|E| from the same start vector: the mixed
     solver (low-precision H·v + an outer Rayleigh-Ritz loop whose H·v is FP64 emulated
-    with float pairs, and again with true FP64 H·v there) and, with --tte-fp64, plain
+    on the tensor cores, and again with true FP64 H·v there) and, with --tte-fp64, plain
     FP64 Lanczos."""
     import torch
     from paper_0707_0159_gb300 import dmrg2d, synth

@@ -215,7 +215,7 @@ int dmrg2d_lanczos_ground(const dmrg2d_ops* ops, const dmrg2d_solver_opts* opts,
 /* Lowest eigenpair of the symmetric tridiagonal matrix T (diagonal alpha[0..k),
  * off-diagonal beta[0..k-1)) — the small eigenproblem inside every Lanczos solve of the
  * superblock (the paper's exact diagonalisation names no eigensolver).  One block: the
- * eigenvalue by multisection on Sturm counts (257 points per round), the eigenvector by
+ * eigenvalue by multisection on Sturm counts (33-fold per round), the eigenvector by
  * the twisted factorisation of T - theta (inverse iteration as the fallback).
  *   alpha, beta: device, k doubles each (beta[k-1] is the coupling of the Krylov space to
  *   the next Lanczos vector: it enters only the residual estimate out[1]).

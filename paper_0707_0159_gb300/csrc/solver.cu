@@ -614,9 +614,9 @@ k_cg_direction(float* __restrict__ p, const float* __restrict__ r, const double*
 }
 
 // ---- lowest eigenpair of the Lanczos tridiagonal T_k (diag alpha, off-diag beta) ----
-// One block.  The eigenvalue by multisection: every thread evaluates the Sturm count
-// (the number of negative pivots of the LDL^T factorisation of T - x, Sylvester's law of
-// inertia) at its own point of the current interval, which shrinks 257-fold per round.
+// One block.  The eigenvalue by multisection: every lane of a warp evaluates the Sturm count
+// (sign changes of the leading minors of T - x) at its own point of the current interval,
+// which shrinks 33-fold per round.
 // The eigenvector by the twisted factorisation of T - theta (Dhillon and Parlett): the
 // top-down LDL^T (thread 0) and bottom-up UDU^T (thread 32) pivots give the twist
 // index r with the smallest |gamma_r|, and z solves (T - theta) z = gamma_r e_r with
