@@ -63,11 +63,17 @@ enum {
   DMRG2D_BF16 = 2,   /* v bf16 (uint16 bits), y float; tcgen05 kind::f16, FP32 acc  */
   DMRG2D_FP32 = 3,   /* v float, y float; FP32 FMA on CUDA cores                      */
   DMRG2D_FP64X = 4,  /* v, y double; FP64 emulated for the mixed solver's residuals: the
-                        entries of v and of the operator blocks as integers of 52 bits
+                        entries of v and of the operator blocks as integers of 60 bits
                         below the largest entry of their row (of H_l, H_r) or line (of
-                        V), multiplied exactly in FP16 digits on the tensor cores;
-                        products below 2^-52 of the largest one are left out.  Scalar
-                        moves in FP64.  A non-finite entry gives NaN                 */
+                        V), multiplied in FP16 digits on the tensor cores, the sums in
+                        64-bit integers.  The error of an output is about 2^-52 of the
+                        product of its row's and its line's largest entries (K up to 256,
+                        twice that for each doubling of K), so of the size of FP64's own
+                        where outputs are of the size of the rest; components far smaller
+                        than the rest of their line (a symmetry sector with 2^-40 of the
+                        weight) keep that absolute error and lose relative accuracy:
+                        DMRG2D_FP64 keeps it.  Scalar moves in FP64.  A non-finite entry
+                        gives NaN                                                      */
   DMRG2D_BF16X3 = 5  /* split BF16: v = [v_hi | v_lo], 2 n_vec bf16 values with
                         v_hi = bf16(x), v_lo = bf16(x - v_hi) (dmrg2d_convert_input);
                         y float; three BF16 tensor-core products into FP32,

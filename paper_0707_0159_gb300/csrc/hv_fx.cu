@@ -1,22 +1,28 @@
 // FP64X: H·v with FP64 vectors and operators on the FP16 tensor cores, exactly split.
 //
 // Every operand row (128 long indices of V, up to 64 segment indices of an operator) is
-// scaled by a power of two so that its entries are 53-bit integers, and each integer is
-// written as seven balanced base-256 digits, which FP16 holds exactly.  Products of digits
-// summed over 128 K stay below 2^24, so the tensor cores' FP32 accumulators are exact: the
-// 28 products of digits i, j with i + j = d <= 6 go into seven accumulators (one per
-// d), which are then added into one 64-bit integer per output.  Rounding happens when an
-// entry is cut to its row's scale (2^-52 of the row's largest entry), by the products left
-// out (i + j > 6, about 2^-52 of the largest product), when a group of stages is added
-// (2^-51 of the largest product) and in the final conversion.
+// scaled by a power of two so that its entries are 61-bit integers, and each integer is
+// written as eight balanced base-256 digits, which FP16 holds exactly.  Products of digits
+// summed over 128 K stay within 2^24, so the tensor cores' FP32 accumulators are exact: the
+// 36 products of digits i, j with i + j = d <= 7 go into eight accumulators (one per d),
+// which are then added into one 64-bit integer per output.  Rounding happens when an entry
+// is cut to its row's scale (2^-60 of the row's largest entry), by the products left out
+// (i + j > 7, about 2^-60 of the product of the two rows' largest entries), when a group of
+// stages is added (2^-54 of the two scales' product for K up to 256, twice that for each
+// doubling of K) and in the final conversion.
+// With seven digits, 53-bit integers and 28 products (9.65 ms on the dense superblock below)
+// the error was larger than float pairs' where the operator's rows and the vector are uneven,
+// as ground states are: 1.9e-14 against 1.1e-14 on that of a 2 x 8 Hubbard ladder, m = 40.
+// It is now 1.0e-15 there (FP64: 2.8e-16).  An entry far below the largest of its row is still
+// held in fewer bits than by itself.
 //
 // Two passes over Y (longplan.h).  A CTA per SM walks its items; per stage of 32 K
 //   warps 0-7   load FP64 entries of V, keep a scale for each row (the largest exponent so
 //               far and one bit) and write their digits into shared memory (two stages);
 //   warps 8-11  do the same for the operator (scales known from the build);
 //   warp 12     issues the tcgen05.mma (M = 128 long indices, K = 16).  The operator's digits
-//               lie one after another along N, so digit i of V meets all digits j <= 6 - i in
-//               one instruction (two above N = 256) that adds to diagonals i .. 6;
+//               lie one after another along N, so digit i of V meets all digits j <= 7 - i in
+//               one instruction (two above N = 256) that adds to diagonals i .. 7;
 //   warps 16-23 add the diagonals from tensor memory to their integers, after at most four
 //               stages or when a scale has grown (the integers are then shifted).
 //
@@ -25,14 +31,15 @@
 // 45 % of the integer pipe: three warps on an SM quarter do not hide its latencies), and the
 // addition of the diagonals (5000-8000 cycles a group, during which no MMA runs).  The MMAs
 // took 1800 cycles a stage with a guard predicate on each (84 to issue one); issued in a block
-// of one elected lane they take half (dense m = 128 10.40 -> 9.65 ms).  Measured against float pairs on the FP32 pipes (12
-// FP32 operations per product, pieces of 64 x 64):
-//   3-leg Hubbard dense, m = 128          73.6 -> 9.65 ms (25 TFLOP/s), error 1.7e-13 -> 3.3e-14
-//   4-leg Heisenberg sectors, m = 512     16.8 -> 1.89 ms,              error 2.6e-13 -> 1.5e-14
-//   3-leg Hubbard sectors, m = 256        44.7 -> 1.78 ms
-// Tried and left out: 8 instead of 12 conversion warps, one warp role for conversion and
-// addition (17 ms), the swizzled operand layouts (11.0 ms), one accumulation per stage
-// (17.8 ms), one MMA per pair of digits (13.3 ms).
+// of one elected lane they take half (dense m = 128 10.40 -> 9.65 ms).  (Cycles with seven
+// digits.)  Measured against float pairs on the FP32 pipes (12 FP32 operations per product,
+// pieces of 64 x 64):
+//   3-leg Hubbard dense, m = 128          73.6 -> 11.3 ms (21 TFLOP/s), error 1.7e-13 -> 2.5e-15
+//   4-leg Heisenberg sectors, m = 512     16.8 -> 2.23 ms,              error 2.6e-13 -> 8.6e-16
+//   3-leg Hubbard sectors, m = 256        44.7 -> 1.81 ms
+// Tried with seven digits and left out: 8 instead of 12 conversion warps, one warp role for
+// conversion and addition (17 ms), the swizzled operand layouts (11.0 ms), one accumulation
+// per stage (17.8 ms), one MMA per pair of digits (13.3 ms).
 #include <algorithm>
 #include <type_traits>
 
@@ -53,7 +60,7 @@ constexpr int FX_THREADS = 32 * (FX_EPI0 + FX_EPI);
 // registers per thread of the conversion, MMA and epilogue warpgroups; the launch gives
 // 768 x 80 = 61440, they take 128 (3 x 64 + 48 + 2 x 120) = 61440
 constexpr int FX_R_CONV = 64, FX_R_MMA = 48, FX_R_EPI = 120;
-constexpr int FX_S = 7;                                // digits = diagonals
+constexpr int FX_S = 8;                                // digits = diagonals
 constexpr int FX_K = 32;                               // K per stage
 constexpr uint32_t FX_A = FX_LONG * FX_K * 2, FX_B = LP_ROWS * FX_K * 2;  // one digit, bytes
 constexpr uint32_t FX_STAGE = FX_S * (FX_A + FX_B);
@@ -65,7 +72,7 @@ constexpr int FX_EMIN = 64;    // exponent fields below this are treated as zero
 // a scale (exponent field) above the 20 bits of a high word's mantissa, all ones
 // (2048, above every finite exponent and one bit: the row has an Inf or NaN)
 __device__ __forceinline__ uint32_t scale_word(uint32_t e) { return e << 20 | 0xfffffu; }
-// Digits of (53-bit mantissa >> (scale - exponent)) with the sign of d, for four values, packed
+// Digits of (53-bit mantissa 2^8 >> (scale - exponent)) with the sign of d, for four values, packed
 // in pairs; E[i]: the scale as scale_word; out[i * stride8]: digit i (0 = most significant)
 // as 4 halves.
 __device__ __forceinline__ void digits4(const double* d, const uint32_t (&E)[4], uint2* out,
@@ -87,11 +94,11 @@ __device__ __forceinline__ void digits4(const double* d, const uint32_t (&E)[4],
     const uint32_t h = (uint32_t)__double2hiint(d[i]);
     // scale - exponent: the mantissa bits of h only lower the difference of the low 20 bits.
     // shr takes shifts above 63 as 64
-    const uint32_t sh = (E[i] - (h & 0x7fffffffu)) >> 20;
-    uint64_t m = ((uint64_t)((h & 0xfffffu) | 0x100000u) << 32) | (uint32_t)__double2loint(d[i]);
+    const uint32_t sh = (E[i] - (h & 0x7fffffffu)) >> 20, l = (uint32_t)__double2loint(d[i]);
+    uint64_t m = ((uint64_t)__funnelshift_l(l, (h & 0xfffffu) | 0x100000u, 8) << 32) | (l << 8);
     asm("shr.u64 %0, %0, %1;" : "+l"(m) : "r"(sh));
-    // the digit bias 0x80 in every byte; byte 7 = 0x64 (FP16 1024 + byte)
-    const uint64_t q = m + 0x6480808080808080ull;
+    // the digit bias 0x80 in every byte
+    const uint64_t q = m + 0x8080808080808080ull;
     lo[i] = (uint32_t)q;
     hi[i] = (uint32_t)(q >> 32);
   }
@@ -102,16 +109,11 @@ __device__ __forceinline__ void digits4(const double* d, const uint32_t (&E)[4],
     return *reinterpret_cast<const uint32_t*>(&r);
   };
 #pragma unroll
-  for (int i = 0; i < 3; ++i) {
-    const int p = 2 - i, sel = 0x7030 | ((4 + p) << 8) | p;
-    *out = make_uint2(fin(__byte_perm(hi[0], hi[1], sel), 0), fin(__byte_perm(hi[2], hi[3], sel), 1));
-    out += stride8;
-  }
-#pragma unroll
-  for (int j = 0; j < 2; ++j) {  // bytes 3, 2 then 1, 0 of the low words
-    // {a.hi, b.hi, a.lo, b.lo} of the byte pair
-    const uint32_t x0 = __byte_perm(lo[0], lo[1], j == 0 ? 0x6273 : 0x4051);
-    const uint32_t x1 = __byte_perm(lo[2], lo[3], j == 0 ? 0x6273 : 0x4051);
+  for (int j = 0; j < 4; ++j) {  // bytes 3, 2 then 1, 0 of the high, then the low words
+    const uint32_t* w = j < 2 ? hi : lo;
+    // {a.hi, b.hi, a.lo, b.lo} of the byte pair; 0x64 above a byte: FP16 1024 + byte
+    const uint32_t x0 = __byte_perm(w[0], w[1], (j & 1) == 0 ? 0x6273 : 0x4051);
+    const uint32_t x1 = __byte_perm(w[2], w[3], (j & 1) == 0 ? 0x6273 : 0x4051);
     *out = make_uint2(fin(__byte_perm(x0, 0x64646464u, 0x4140), 0),
                       fin(__byte_perm(x1, 0x64646464u, 0x4140), 1));
     out += stride8;
@@ -417,7 +419,7 @@ __global__ void __launch_bounds__(FX_THREADS, 1) hv_fx_kernel(const FxParams p) 
                 const uint64_t a = a0 + ((i * FX_A + k * AK) >> 4), bb = b0 + ((k * 256) >> 4);
                 const uint32_t dt = tmem + n * i, acc = k > 0 || i > 0 || !fresh;
                 umma_t<1>(dt, a, bb, id | (min(w, 256u) >> 3) << 17, acc);
-                if (i < 3 && w > 256)  // N = 48 or 64: the columns above 256
+                if (i < 4 && w > 256)  // N = 48 or 64: the columns above 256
                   umma_t<1>(dt + 256, a, bb + ((256 / 8 * FX_K * 16) >> 4),
                             id | ((w - 256) >> 3) << 17, acc);
               }
@@ -450,7 +452,7 @@ __global__ void __launch_bounds__(FX_THREADS, 1) hv_fx_kernel(const FxParams p) 
               const int eb = p.opE[sg.e0 + it.s0 + j0 + j];
               const bool bad = E == 2048 || eb == 2047;  // Inf or NaN
               yp[(long long)sg.ld * j] =
-                  bad ? nanv : scaled(acc[j], E + eb + sg.head + 56 - 2 * 1075);
+                  bad ? nanv : scaled(acc[j], E + eb + sg.head + 68 - 2 * 1083);
             }
         } else {
           double* yp = p.y + sg.base + j1 + (long long)sg.ld * x;
@@ -459,7 +461,7 @@ __global__ void __launch_bounds__(FX_THREADS, 1) hv_fx_kernel(const FxParams p) 
             if (j < nj) {
               const int eb = p.opE[sg.e0 + it.s0 + j0 + j];
               const bool bad = E == 2048 || eb == 2047;  // Inf or NaN
-              yp[j] += bad ? nanv : scaled(acc[j], E + eb + sg.head + 56 - 2 * 1075);
+              yp[j] += bad ? nanv : scaled(acc[j], E + eb + sg.head + 68 - 2 * 1083);
             }
           // the segment's padding rows, after its last index
           if (it.s0 + j0 + nj == sg.dim && (half == 1 || it.cnt <= 32))
@@ -510,15 +512,16 @@ __global__ void __launch_bounds__(FX_THREADS, 1) hv_fx_kernel(const FxParams p) 
             if (go) tmem_ld8(d + 1 < FX_S ? tc + (d + 1) * N + 8 * h : tc + 8 * h + 8, nxt);
 #pragma unroll
             for (int j = 0; j < 8; ++j) {
-              // weight 2^(40 - 8 d); d = 6 is rounded to the unit.  |sum| < 2^22 for d <= 2
-              // (the leading digits are at most 33): the cheap conversion
+              // weight 2^(44 - 8 d); d = 6 and 7 are rounded to the unit.  |sum| < 2^22 for
+              // d <= 2 (the leading digits are at most 33): the cheap conversion
               constexpr float magic = 12582912.f;  // 1.5 * 2^23: the integer in the low bits
               const float x = __uint_as_float(cur[j]);
               int a = d < 3 ? __float_as_int(x + magic) - 0x4B400000 : __float2int_rn(x);
-              if (d == 6) a = (a + 128) >> 8;
-              constexpr int W[FX_S] = {0, 0, 1 << 24, 1 << 16, 1 << 8, 1, 1};
+              if (d == 6) a = (a + 8) >> 4;
+              if (d == 7) a = (a + 2048) >> 12;
+              constexpr int W[FX_S] = {0, 0, 1 << 28, 1 << 20, 1 << 12, 1 << 4, 1, 1};
               if (d < 2)
-                acc[8 * h + j] += (long long)((unsigned long long)(unsigned)(d == 0 ? a * 256 : a) << 32);
+                acc[8 * h + j] += (long long)((unsigned long long)(unsigned)(a * (d == 0 ? 4096 : 16)) << 32);
               else
                 asm("mad.wide.s32 %0, %1, %2, %0;" : "+l"(acc[8 * h + j]) : "r"(a), "r"(W[d]));
             }

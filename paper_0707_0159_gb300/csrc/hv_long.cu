@@ -496,8 +496,8 @@ int lp_finalise(dmrg2d_ops* ops, LongPlan* L, cudaStream_t s) {
           L->units[ps].push_back({k.op + k0, k.v_off + k0, k.kdim, std::min(8, k.kdim - k0)});
       }
       sg.ue = (int)L->units[ps].size();
-      sg.head = 0;  // 64-bit sums of K products below 2^50 each
-      while ((kt >> sg.head) > 4096) ++sg.head;
+      sg.head = 0;  // 64-bit sums of K products below 2^54 each
+      while ((kt >> sg.head) > 256) ++sg.head;
     }
     L->items[ps] = cut(L, ps, LP_ROWS, 1, [](int cnt) { return 64 * (8 / row_groups(cnt)); });
     L->items32[ps] = cut(L, ps, LP_ROWS, 4, long_of32);

@@ -25,7 +25,7 @@ struct LSeg {
   int kb, ke;      // operator blocks ks[kb..ke)
   int ub, ue;      // the same blocks as units[ub..ue)
   int e0;          // first entry of the segment's operator rows in opE
-  int head;        // extra exponent bits of the operator side (K above 8192)
+  int head;        // extra exponent bits of the operator side (K above 256)
 };
 struct LK {
   long long op;    // element offset of the block (row-major dim x kdim)
