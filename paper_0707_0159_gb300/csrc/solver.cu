@@ -1894,16 +1894,18 @@ static int mixed_outer(Ctx& C, const dmrg2d_solver_opts* o, double* x, double* e
     }));
     // The next step is in the queue before the host waits for the one before it; the device
     // decides when to stop (a step after that changes nothing).
+    int replays = 0;
     for (int it = 0; it < o->inner_iter; ++it) {
       D2_CUDA(cudaGraphLaunch(step.exec, C.s));
+      ++replays;
       D2_CUDA(cudaEventRecord(step.done[it & 1], C.s));
       if (it == 0) continue;
       D2_CUDA(cudaEventSynchronize(step.done[(it - 1) & 1]));
       if (*(volatile double*)C.hscal != 0.0) break;
     }
     D2_CUDA(cudaStreamSynchronize(C.s));
-    C.st->n_hv_low += (int)C.hscal[CG_STEPS - CG_STOP];
-    C.st->iters += (int)C.hscal[CG_STEPS - CG_STOP];
+    C.st->n_hv_low += replays;  // a step after the last one runs its H·v too
+    if (replays > 0) C.st->iters += (int)C.hscal[CG_STEPS - CG_STOP];
     k_f32_to_f64<<<g, VT, 0, C.s>>>(t32, t, n);
     D2_CUDA(cudaGetLastError());
     // ---- orthonormalise t against U and extend the subspace ----
