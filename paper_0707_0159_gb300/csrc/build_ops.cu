@@ -590,6 +590,7 @@ extern "C" int dmrg2d_profile_stop(dmrg2d_ops* ops, double* total_ms, int* launc
 extern "C" void dmrg2d_free_ops(dmrg2d_ops* ops) {
   if (!ops) return;
   prof_clear(ops);
+  for (int i = 0; i < ops->host_kept; ++i) cudaFreeHost(ops->host_slot[i]);
   lp_release(ops->lp);
   sec_release(ops);
   tc_release(ops);

@@ -6,6 +6,7 @@
 #include <cuda_bf16.h>
 #include <cstdint>
 #include <cstdio>
+#include <mutex>
 #include <string>
 #include <vector>
 
@@ -79,6 +80,8 @@ struct DeviceOps {
 
 struct LongPlan;
 
+constexpr int HOST_SLOTS = 8;  // pinned host slots an ops object keeps (solver.cu)
+
 }  // namespace dmrg2d
 
 struct dmrg2d_ops {
@@ -110,6 +113,10 @@ struct dmrg2d_ops {
   mutable std::vector<std::pair<cudaEvent_t, cudaEvent_t>> prof_ev;
   mutable size_t prof_used = 0;
   mutable bool prof_on = false;
+  // pinned host memory of the solves that are not running, 64 doubles each
+  mutable std::mutex host_mu;
+  mutable double* host_slot[dmrg2d::HOST_SLOTS] = {};
+  mutable int host_kept = 0;
 };
 
 namespace dmrg2d {

@@ -16,7 +16,6 @@
 #include <algorithm>
 #include <chrono>
 #include <cmath>
-#include <mutex>
 #include <vector>
 
 #include <cooperative_groups.h>
@@ -1466,47 +1465,30 @@ int dmalloc(DevBuf& b, size_t bytes) {
 }
 
 // 64 pinned doubles for the scalars a solve reads back.  cudaMallocHost and cudaFreeHost took
-// 270 us of every call (a quarter of the first Lanczos steps of a small superblock), so up to
-// PINNED_KEPT slots are kept between calls: one per solve running at a time, under a mutex,
-// given back after the solve's stream has finished.
-constexpr int PINNED_KEPT = 8;
+// 270 us of every call (a quarter of the first Lanczos steps of a small superblock), so an ops
+// object keeps up to HOST_SLOTS of them between calls: one per solve running at a time, under
+// its mutex, given back after the solve's stream has finished and freed with the object.  (None
+// outlives it: an address kept beyond a device reset may be a caller's new buffer by then.)
 struct PinnedSlot {
+  const dmrg2d_ops* ops;
+  cudaStream_t s;
   double* p = nullptr;
-  cudaStream_t s = nullptr;
-  static std::vector<double*>& kept() {
-    static std::vector<double*> v;
-    return v;
-  }
-  static std::mutex& mu() {
-    static std::mutex m;
-    return m;
-  }
-  int take(cudaStream_t stream) {
-    s = stream;
+  PinnedSlot(const dmrg2d_ops* o, cudaStream_t stream) : ops(o), s(stream) {}
+  int take() {
     {
-      std::lock_guard<std::mutex> lk(mu());
-      if (!kept().empty()) {
-        p = kept().back();
-        kept().pop_back();
-      }
+      std::lock_guard<std::mutex> lk(ops->host_mu);
+      if (ops->host_kept > 0) p = ops->host_slot[--ops->host_kept];
     }
-    if (p) {  // still pinned (the device may have been reset meanwhile)?
-      cudaPointerAttributes a;
-      if (cudaPointerGetAttributes(&a, p) == cudaSuccess && a.type == cudaMemoryTypeHost)
-        return DMRG2D_OK;
-      cudaGetLastError();
-      p = nullptr;
-    }
-    D2_CUDA(cudaHostAlloc((void**)&p, sizeof(double) * 64, cudaHostAllocPortable));
+    if (!p) D2_CUDA(cudaHostAlloc((void**)&p, sizeof(double) * 64, cudaHostAllocPortable));
     return DMRG2D_OK;
   }
   ~PinnedSlot() {
     if (!p) return;
     const bool idle = cudaStreamSynchronize(s) == cudaSuccess;  // no copy into it is in flight
     if (idle) {
-      std::lock_guard<std::mutex> lk(mu());
-      if ((int)kept().size() < PINNED_KEPT) {
-        kept().push_back(p);
+      std::lock_guard<std::mutex> lk(ops->host_mu);
+      if (ops->host_kept < HOST_SLOTS) {
+        ops->host_slot[ops->host_kept++] = p;
         return;
       }
     }
@@ -1973,8 +1955,8 @@ extern "C" int dmrg2d_lanczos_ground(const dmrg2d_ops* ops, const dmrg2d_solver_
                      {&C.scal, sizeof(double) * 64},
                      {&C.lo, low ? (o.precision == DMRG2D_BF16 ? 2 : 4) * (size_t)C.n : 0},
                      {&C.y32, low ? sizeof(float) * (size_t)C.n : 0}}));
-  PinnedSlot pinned;
-  D2_TRY(pinned.take(C.s));
+  PinnedSlot pinned(ops, C.s);
+  D2_TRY(pinned.take());
   C.hscal = pinned.p;
   int st;
   double energy = 0.0;
@@ -2043,7 +2025,6 @@ extern "C" int dmrg2d_tridiag_lowest(const double* alpha, const double* beta, in
 // runtime for the array's device address once per device and hands that to the kernels.
 static __device__ __align__(256) double g_noalloc_scratch[DMRG2D_NOALLOC_SCRATCH_DOUBLES];
 
-#include <mutex>
 
 namespace dmrg2d {
 namespace {
@@ -2389,8 +2370,8 @@ extern "C" int dmrg2d_davidson_ground(const dmrg2d_ops* ops, const dmrg2d_davids
                      {&C.scal, sizeof(double) * 64},
                      {&C.lo, low ? (o.precision == DMRG2D_BF16 ? 2 : 4) * (size_t)C.n : 0},
                      {&C.y32, low ? sizeof(float) * (size_t)C.n : 0}}));
-  PinnedSlot pinned;
-  D2_TRY(pinned.take(C.s));
+  PinnedSlot pinned(ops, C.s);
+  D2_TRY(pinned.take());
   C.hscal = pinned.p;
   D2_TRY(sec_zero_padding(ops, x_inout, C.s));
   double energy = 0.0, resid = 0.0;
