@@ -35,10 +35,19 @@ int vgrid(int64_t n) {
   return (int)(g < RED_BLOCKS ? (g < 1 ? 1 : g) : RED_BLOCKS);
 }
 
-// CTAs of a reduction over FP64 vectors: three per SM.  Every CTA ends in a tree of FP64
-// additions at 2 per clock and SM (eight of them in k_multidot_partial: 87 us with 1216 CTAs on
-// 3.4e6 elements, 74 with 456).
-int rgrid(int64_t n) { return std::min(vgrid(n), 456); }
+// CTAs of a pass that ends in a reduction: `per_sm` on each SM (at most RED_BLOCKS in all).
+// Every CTA costs a tree of FP64 additions at 2 per clock and SM, which counts on short vectors
+// (k_multidot_partial, eight trees: 49 us with 1216 CTAs on 3.4e6 elements, 31 with 456); long
+// ones need the bytes in flight of more CTAs where a thread's loads are few.  Microseconds on
+// 152 SMs, FP32 unless said, n = 3.4e6 / 1.7e7 / 2.7e8:
+//   CTAs           304                456                608                1216
+//   k_cg_dots      14.5 / 53 / 661    15.3 / 45 / 513    16.4 / 43 / 471    21.0 / 51 / 516
+//   k_cg_update    18.5 / 84 / 1157   18.4 / 78 / 1065   18.0 / 78 / 1179   20.5 / 79 / 1149
+//   k_dot..32      12.3 / 47 / 592    12.3 / 38 / 436    12.3 / 34 / 369    14.3 / 32 / 333
+//   k_lz_axpy2..   16.4 / 128 / 1846  14.9 / 93 / 1290   14.4 / 76 / 1029   16.4 / 56 / 694
+//   FP64 dot       14.4 / 58          14.4 / 50          15.3 / 48          16.4 / 50
+constexpr int64_t LONG_VECTOR = 1 << 23;
+int red_grid(int64_t n, int sms, int per_sm) { return std::min(vgrid(n), per_sm * sms); }
 
 __device__ __forceinline__ double warp_sum(double v) {
 #pragma unroll
@@ -429,10 +438,6 @@ __global__ void k_scale_to32(float* __restrict__ q, const TI* __restrict__ in,
 // alone: the host launches a step before it has seen the result of the one before.
 enum { CG_XQ = 40, CG_PQ, CG_A, CG_RR, CG_RR1, CG_BETA, CG_THETA, CG_RR0, CG_STOP, CG_STEPS,
        CG_COUNT };  // CG_COUNT: two unsigned arrival counters
-
-// 304 CTAs (two per SM): every CTA costs a tree of FP64 additions at GB300's FP64 rate (with
-// 1216 it was half of a pass's time), and float4 loads keep enough bytes in flight
-int cg_grid(int64_t n) { return (int)std::max<int64_t>(1, std::min<int64_t>(304, n / (4 * VT))); }
 
 // true in the CTA that arrives last; the partial sums written before are then visible
 __device__ bool last_block(unsigned* count) {
@@ -1322,6 +1327,20 @@ struct Ctx {
   std::vector<std::pair<cudaEvent_t, cudaEvent_t>> ev;
   size_t ev_used = 0;
   bool timing = true;
+  int sms = 1;  // of the current device
+
+  Ctx() {
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess ||
+        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
+      sms = 1;
+  }
+  // CTAs of the FP64 reductions, and of the FP32 ones (red_grid)
+  int rgrid() const { return red_grid(n, sms, 3); }
+  int dot32_grid() const { return red_grid(n, sms, n < LONG_VECTOR ? 3 : 8); }
+  int axpy32_grid() const { return red_grid(n, sms, n < LONG_VECTOR ? 4 : 8); }
+  int cg_dots_grid() const { return red_grid((n + 3) / 4, sms, n < LONG_VECTOR ? 2 : 4); }
+  int cg_update_grid() const { return red_grid((n + 3) / 4, sms, 3); }
 
   int hv(int prec, const double* x, double* y) {
     cudaEvent_t a = nullptr, b = nullptr;
@@ -1392,14 +1411,14 @@ struct Ctx {
 
   // *out (device) = a . b
   int dot(const double* a, const double* b, double* out) {
-    const int g = rgrid(n);
+    const int g = rgrid();
     k_dot_partial<<<g, VT, 0, s>>>(a, b, n, part);
     k_reduce<<<1, VT, 0, s>>>(part, g, out, 0);
     D2_CUDA(cudaGetLastError());
     return DMRG2D_OK;
   }
   int nrm(const double* a, double* out) {
-    const int g = rgrid(n);
+    const int g = rgrid();
     k_dot_partial<<<g, VT, 0, s>>>(a, a, n, part);
     k_reduce<<<1, VT, 0, s>>>(part, g, out, 1);
     D2_CUDA(cudaGetLastError());
@@ -1407,7 +1426,7 @@ struct Ctx {
   }
   // h[0..k) = Q[0..k) . w
   int multidot(const double* Q, int64_t stride, int k, const double* w, double* h) {
-    const int g = rgrid(n);
+    const int g = rgrid();
     dim3 grid(g, (k + MD_CHUNK - 1) / MD_CHUNK);
     k_multidot_partial<<<grid, VT, 0, s>>>(Q, stride, k, w, n, part);
     k_reduce<<<k, VT, 0, s>>>(part, g, h, 0);
@@ -1431,9 +1450,8 @@ struct Ctx {
   }
   // CTAs of k_lz_step for this vector length; 0 when it does not fit (or no cooperative launch)
   int lz_grid() const {
-    int dev = 0, sms = 0, coop = 0;
+    int dev = 0, coop = 0;
     if (cudaGetDevice(&dev) != cudaSuccess ||
-        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
         cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev) != cudaSuccess || !coop)
       return 0;
     if (n > (int64_t)sms * LZ_CHUNK) return 0;
@@ -1642,7 +1660,7 @@ int lanczos_lo(Ctx& C, int prec, double* x, int max_iter, int kdim, double tol, 
                      {&scr, 6 * kd}}));
   float* w = C.y32;  // H~ q_j lands here and is orthogonalised in place
   double* out3 = C.scal;
-  const int g = vgrid(n), gr = rgrid(n);
+  const int g = vgrid(n), gd = C.dot32_grid(), ga = C.axpy32_grid();
   auto start_from_x = [&]() -> int {
     D2_TRY(C.nrm(x, C.scal + 3));
     k_scale_to32<double><<<g, VT, 0, C.s>>>(Q, x, C.scal + 3, C.lo, prec, n);
@@ -1657,11 +1675,11 @@ int lanczos_lo(Ctx& C, int prec, double* x, int max_iter, int kdim, double tol, 
   while (true) {
     float* qj = Q + (int64_t)j * n;
     D2_TRY(C.hv_lo(prec));  // w = H~ q_j (its H~-format copy is in C.lo)
-    k_dot_partial32<<<gr, VT, 0, C.s>>>(qj, w, n, C.part);
-    k_reduce<<<1, VT, 0, C.s>>>(C.part, gr, alpha + j, 0);
-    k_lz_axpy2_nrm32<<<gr, VT, 0, C.s>>>(w, qj, j > 0 ? qj - n : nullptr, alpha + j,
+    k_dot_partial32<<<gd, VT, 0, C.s>>>(qj, w, n, C.part);
+    k_reduce<<<1, VT, 0, C.s>>>(C.part, gd, alpha + j, 0);
+    k_lz_axpy2_nrm32<<<ga, VT, 0, C.s>>>(w, qj, j > 0 ? qj - n : nullptr, alpha + j,
                                         j > 0 ? beta + j - 1 : nullptr, n, C.part);
-    k_reduce<<<1, VT, 0, C.s>>>(C.part, gr, beta + j, 1);
+    k_reduce<<<1, VT, 0, C.s>>>(C.part, ga, beta + j, 1);
     for (int pass = 0; pass < gs_passes; ++pass) {  // CGS against q_0..q_j
       dim3 grid(g, (j + 1 + MD_CHUNK - 1) / MD_CHUNK);
       k_multidot_partial32<<<grid, VT, 0, C.s>>>(Q, n, j + 1, w, n, C.part);
@@ -1865,9 +1883,8 @@ static int mixed_outer(Ctx& C, const dmrg2d_solver_opts* o, double* x, double* e
     if (!step.exec) D2_TRY(step.capture(C, [&]() -> int {
       // one CG step: y32 = H~ p, the fused vector passes, the stop flag to the pinned mirror
       D2_TRY(C.hv_lo(prec, nullptr, nullptr, false));  // counted per replay
-      const int cg = cg_grid(n);
-      k_cg_dots<<<cg, VT, 0, C.s>>>(C.y32, p32, x32, sc, n, C.part);
-      k_cg_update<<<cg, VT, 0, C.s>>>(C.y32, p32, x32, t32, r32, sc, n, C.part);
+      k_cg_dots<<<C.cg_dots_grid(), VT, 0, C.s>>>(C.y32, p32, x32, sc, n, C.part);
+      k_cg_update<<<C.cg_update_grid(), VT, 0, C.s>>>(C.y32, p32, x32, t32, r32, sc, n, C.part);
       k_cg_direction<<<vgrid((n + 3) / 4), VT, 0, C.s>>>(p32, r32, sc, C.lo, prec, n);
       D2_CUDA(cudaGetLastError());
       D2_CUDA(cudaMemcpyAsync(C.hscal, sc + CG_STOP, sizeof(double) * 2, cudaMemcpyDeviceToHost,
