@@ -205,7 +205,8 @@ typedef struct dmrg2d_solver_stats {
   int outer;           /* FP64 outer iterations (mixed)                             */
   int n_hv_fp64;       /* FP64 H·v calls                                            */
   int n_hv_low;        /* low-precision H·v calls (mixed: a correction solve that stops
-                          before inner_iter may have run one after its last step)    */
+                          before inner_iter may have run one after its last step, on
+                          vectors below 2^23 elements)                              */
   double resid;        /* final ||H x - theta x|| (FP64)                            */
   double hv_ms;        /* device time spent in H·v launches (CUDA events)           */
   double elapsed_ms;   /* wall time of the call                                     */

@@ -435,7 +435,7 @@ __global__ void k_scale_to32(float* __restrict__ q, const TI* __restrict__ in,
 // With float4 accesses and one step queued ahead of the host, a step of the mixed solve on the
 // 4-leg Heisenberg sectors of m = 256 (n = 3.4e6) went from 145 to 110 us, 79 of them H~ p.
 // Once a step has met p.q <= 0 or r.r <= 1e-8 r0.r0, CG_STOP makes later steps leave t and r
-// alone: the host launches a step before it has seen the result of the one before.
+// alone: the host may launch a step before it has seen the result of the one before.
 enum { CG_XQ = 40, CG_PQ, CG_A, CG_RR, CG_RR1, CG_BETA, CG_THETA, CG_RR0, CG_STOP, CG_STEPS,
        CG_COUNT };  // CG_COUNT: two unsigned arrival counters
 
@@ -1891,15 +1891,19 @@ static int mixed_outer(Ctx& C, const dmrg2d_solver_opts* o, double* x, double* e
                               C.s));
       return DMRG2D_OK;
     }));
-    // The next step is in the queue before the host waits for the one before it; the device
-    // decides when to stop (a step after that changes nothing).
+    // On short vectors the next step is in the queue before the host waits for the one before
+    // it: 62 instead of 66..70 us a step at n = 1e5..3e5, 127 instead of 129 at 3.4e6.  The device
+    // decides when to stop, and a step after that changes nothing, but its H·v is run for nothing:
+    // on long vectors (a step of 0.3 ms and more, 4.5 ms at n = 2.7e8) that costs more than the
+    // waits (both ways 220 ms at n = 1.7e7).
+    const int ahead = n < LONG_VECTOR ? 1 : 0;
     int replays = 0;
     for (int it = 0; it < o->inner_iter; ++it) {
       D2_CUDA(cudaGraphLaunch(step.exec, C.s));
       ++replays;
       D2_CUDA(cudaEventRecord(step.done[it & 1], C.s));
-      if (it == 0) continue;
-      D2_CUDA(cudaEventSynchronize(step.done[(it - 1) & 1]));
+      if (it < ahead) continue;
+      D2_CUDA(cudaEventSynchronize(step.done[(it - ahead) & 1]));
       if (*(volatile double*)C.hscal != 0.0) break;
     }
     D2_CUDA(cudaStreamSynchronize(C.s));

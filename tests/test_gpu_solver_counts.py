@@ -42,3 +42,13 @@ def test_no_inner_steps(ops):
     _, st, code = solve(ops, inner_iter=0, tol=1e-12)
     assert code == -5
     assert st["n_hv_low"] == 1 and st["iters"] == 1
+
+
+def test_no_step_queued_ahead_on_long_vectors():
+    """n = 18.9e6: no H·v is run after the step that met the stopping test."""
+    mdl = synth.model("hubbard", 3, t=1.0, U=8.0)
+    long_ops = dmrg2d.build_ops(mdl, synth.hubbard_block(64, 3, 5), synth.hubbard_block(72, 3, 6))
+    assert long_ops.info["n_vec"] >= 1 << 23
+    _, st, code = solve(long_ops, inner_iter=500, tol=1e-5)
+    assert code == 0 and st["outer"] >= 1
+    assert st["n_hv_low"] == st["iters"]
