@@ -11,6 +11,7 @@
 
 #include "common.h"
 #include "longplan.h"
+#include "simt_choice.h"
 
 namespace dmrg2d {
 
@@ -238,8 +239,6 @@ hv_simt_small_kernel(const T* __restrict__ v, T* __restrict__ y, const T* __rest
   y[(int64_t)i2 * m1 + gi + ld * ((int64_t)i3 * m4 + gj)] = acc;
 }
 
-int sm_count(const dmrg2d_ops* ops) { return ops->lp ? ops->lp->sms : 1; }
-
 template <typename T>
 int launch(const dmrg2d_ops* ops, const T* v, T* y, const T* HL, const T* HR, const T* C,
            cudaStream_t s) {
@@ -254,50 +253,20 @@ int launch(const dmrg2d_ops* ops, const T* v, T* y, const T* HL, const T* HR, co
   p.Rcol = ops->dev.Rcol;
   p.Cptr = ops->dev.Cptr;
   p.Csrc = ops->dev.Csrc;
-  const int sms = sm_count(ops);
-  auto ctas = [&](int64_t b) {
-    return ((ops->m1 + b - 1) / b) * ops->d * ((ops->m4 + b - 1) / b) * ops->d;
-  };
-  int tb;
-  bool two_pass = false;
-  if (sizeof(T) == 8) {
-    // Every kernel runs at the FP64 pipe's rate, so the time is the fullest SM's outputs times
-    // their padded K: pieces of 64, 32, 16 or 8, or the two-pass kernel, which pads nothing
-    // but takes two kernels more and 1.1 of the rate, once it has two items per SM.
-    // (3-leg Heisenberg 250 x 131: pieces of 64 9.63 ms, two-pass 6.13 ms; 2-leg 200 x 200:
-    // pieces of 64 2.53 ms, of 8 1.31 ms; 2-leg Hubbard 40 x 40: 0.99 and 0.34 ms.)
-    auto pad = [](int m, int64_t b) { return (double)((m + b - 1) / b * b) / m; };
-    double best = 0.0;
-    tb = 0;
-    for (int b : {64, 32, 16, 8}) {
-      const int64_t g = ctas(b);
-      const double kpad = std::max(pad(ops->m1, BK), pad(ops->m4, BK));
-      const double cost = (double)((g + sms - 1) / sms) * b * b * kpad;
-      if (!tb || cost < 0.98 * best) {
-        best = cost;
-        tb = b;
-      }
-    }
-    two_pass = (int)ops->lp->items[0].size() >= 2 * sms &&
-               1.1 * (double)ops->n_vec / sms < 0.98 * best;
-  } else {
-    // the largest piece (64, 32 or 16 square) whose grid still gives every SM a CTA; the
-    // two-pass kernel's larger register tiles once they fill nearly half of the SMs (2-leg
-    // 100 x 128, 32 items: 66 us in pieces, 67 two-pass; 2-leg Hubbard 40 x 40, 80 items: 80
-    // and 48 us; 3-leg Heisenberg 250 x 131: 641 and 295 us; 3-leg Hubbard 128 x 128: 12.4
-    // and 5.8 ms)
-    tb = ctas(64) >= sms ? 64 : (ctas(32) >= sms ? 32 : 16);
-    two_pass = 5 * (int)ops->lp->items32[0].size() >= 2 * sms;
-  }
-  const int64_t gx = (int64_t)((ops->m1 + tb - 1) / tb) * ops->d;
-  const int64_t gy = (int64_t)((ops->m4 + tb - 1) / tb) * ops->d;
-  if (!two_pass && (gx > 0x7fffffff || gy > 65535))
+  const int sms = ops->lp->sms;
+  const SimtChoice c =
+      sizeof(T) == 8
+          ? simt_choice_f64(ops->m1, ops->m4, ops->d, sms, (int64_t)ops->lp->items[0].size())
+          : simt_choice_f32(ops->m1, ops->m4, ops->d, sms, (int64_t)ops->lp->items32[0].size());
+  const int tb = c.piece;
+  const int64_t gx = simt_pieces(ops->m1, ops->d, tb), gy = simt_pieces(ops->m4, ops->d, tb);
+  if (!c.two_pass && !simt_grid_fits(ops->m1, ops->m4, ops->d, tb))
     return set_error(DMRG2D_EUNSUPPORTED, "SIMT grid %lld x %lld too large", (long long)gx,
                      (long long)gy);
   dim3 grid((unsigned)gx, (unsigned)gy);
   auto ev = prof_slot(ops);
   if (ev.first) D2_CUDA(cudaEventRecord(ev.first, s));
-  if (two_pass) {
+  if (c.two_pass) {
     if constexpr (sizeof(T) == 8) {
       D2_TRY(lp_launch_f64(ops->lp, v, y, s));
       if (ev.second) D2_CUDA(cudaEventRecord(ev.second, s));
