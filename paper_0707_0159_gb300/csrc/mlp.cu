@@ -590,11 +590,13 @@ int loss_and_gradient(dmrg2d_mlp* M, const float* X, const float* w, const float
   k_grad<<<(M->np + 255) / 256, 256, 0, s>>>(s1, c.blocks, s2, c.splits, s3, c.blocks, H, M->np, M->g);
   D2_CUDA(cudaGetLastError());
   if (loss) {
-    std::vector<double> hp(c.blocks);
-    D2_CUDA(cudaMemcpyAsync(hp.data(), M->part, c.blocks * sizeof(double), cudaMemcpyDeviceToHost, s));
-    D2_CUDA(cudaStreamSynchronize(s));
-    double tot = 0;
-    for (double v : hp) tot += v;
+    double hp[1024], tot = 0;  // no host allocation: batches of any size, 1024 sums at a time
+    for (int b0 = 0; b0 < c.blocks; b0 += 1024) {
+      const int nb = std::min(1024, c.blocks - b0);
+      D2_CUDA(cudaMemcpyAsync(hp, M->part + b0, nb * sizeof(double), cudaMemcpyDeviceToHost, s));
+      D2_CUDA(cudaStreamSynchronize(s));
+      for (int i = 0; i < nb; ++i) tot += hp[i];
+    }
     *loss = (float)(tot / (2.0 * B));
   }
   return DMRG2D_OK;
