@@ -450,7 +450,7 @@ hv_tc_seg_kernel(const __grid_constant__ SMaps maps, const SParams p) {
   // MMAs and stores all left out they took 90 % of their time.  So the operator-block entries
   // of a piece are read by the whole warp, one per lane, while the piece before runs, pieces
   // two ahead; the V tile comes in one box and the operator rows in one or two; and the warps'
-  // loop state stays in uniform registers (elect_one).  3-leg Hubbard sectors, m = 1024, TF32:
+  // loop state is the warp's (elect_one, bcast_uniform).  3-leg Hubbard sectors, m = 1024, TF32:
   // passes 1160 and 1380 us -> 890 and 875 us, H·v 3.23 -> 2.46 ms; 4-leg Heisenberg sectors,
   // m = 256: 74.4 -> 60.5 us.
   // {a_pool, b_row, kdim, neg} in pass 1, {a_col, b_pool, kdim, neg} in pass 2

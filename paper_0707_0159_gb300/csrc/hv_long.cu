@@ -1,17 +1,16 @@
-// Two-pass H·v on CUDA cores (FP64 DFMA, FP32 FFMA) over a LongPlan; the scalar moves; the
-// plan's work lists.
+// Two-pass H·v on CUDA cores over a LongPlan, in FP64 (hv_long_kernel) and FP32
+// (hv_long32_kernel); the scalar moves; the plan's work lists.
 //
-// What bounds it: the FP64 pipe (GB300: 2 DFMA per clock and SM, 1.25 TFLOP/s) or the FP32
-// pipe; a warp instruction costs the same with one active lane as with 32.  So lanes run
-// along the long dimension of V_q (hundreds of indices, whole warps of it skipped at the
-// end), and the short side, a quantum-number segment of any size, is held in registers with
-// its exact extent: each warp owns up to 8 of the item's segment indices, and the loop body
-// is instantiated for 1..8 of them.  K runs over each block's exact extent.  Nothing is
-// padded but the last 64 long indices.
+// What bounds FP64: its pipe (GB300: 2 DFMA per clock and SM, 1.25 TFLOP/s); a warp instruction
+// costs the same with one active lane as with 32.  So lanes run along the long dimension of V_q
+// (hundreds of indices, whole warps of it skipped at the end), and the short side, a
+// quantum-number segment of any size, is held in registers with its exact extent: each warp owns
+// up to 8 of the item's segment indices, and the loop body is instantiated for 1..8 of them.  K
+// runs over each block's exact extent.  Nothing is padded but the last 64 long indices.
 // Measured against one 64 x 64 piece per (row segment x column segment), whose padding was
 // the time (3-leg Hubbard superblock of 25 sectors, 4-leg Heisenberg of 7; moves included):
-//   Hubbard m = 256     FP64 115.6 -> 4.42 ms (1.01 TFLOP/s of 1.25), FP32 7.51 -> 0.51 ms
-//   Heisenberg m = 256  FP64 7.85 -> 4.13 ms,                         FP32 0.55 -> 0.20 ms
+//   Hubbard m = 256     FP64 115.6 -> 4.36 ms (1.02 TFLOP/s of 1.25), FP32 7.51 -> 0.52 ms
+//   Heisenberg m = 256  FP64 7.85 -> 4.10 ms,                         FP32 0.55 -> 0.20 ms
 //   Heisenberg m = 1024 FP64 275 -> 218 ms (1.23 TFLOP/s),            FP32 17.8 -> 7.0 ms
 #include <algorithm>
 
@@ -23,51 +22,49 @@ namespace {
 
 constexpr int LT = 256;  // threads: 8 warps = row groups x groups of 64 long indices
 constexpr int TN_MAX = 512;
+constexpr int BK = 8;    // K per chunk
 
 // row groups of an item: 8 indices per warp at most, the other warps along the long side
 __host__ __device__ inline int row_groups(int cnt) {
   return cnt <= 8 ? 1 : cnt <= 16 ? 2 : cnt <= 32 ? 4 : 8;
 }
 
-template <typename T>
 struct alignas(16) Vec16 {
-  T v[16 / sizeof(T)];
+  double v[2];
 };
 
 // acc[a][b] += O[k][a] * V[k][c + 32 b] for the warp's RA indices
-template <typename T, int RA, int OS, int VS>
-__device__ __forceinline__ void mac_k(T (&acc)[8][2], const T* __restrict__ O,
-                                      const T* __restrict__ V, int k) {
-  constexpr int W = 16 / sizeof(T), NV = (RA + W - 1) / W;
-  const T b0 = V[k * VS], b1 = V[k * VS + 32];
-  Vec16<T> o[NV];
+template <int RA, int OS, int VS>
+__device__ __forceinline__ void mac_k(double (&acc)[8][2], const double* __restrict__ O,
+                                      const double* __restrict__ V, int k) {
+  constexpr int W = 2, NV = (RA + W - 1) / W;
+  const double b0 = V[k * VS], b1 = V[k * VS + 32];
+  Vec16 o[NV];
 #pragma unroll
-  for (int i = 0; i < NV; ++i) o[i] = *reinterpret_cast<const Vec16<T>*>(O + k * OS + i * W);
+  for (int i = 0; i < NV; ++i) o[i] = *reinterpret_cast<const Vec16*>(O + k * OS + i * W);
 #pragma unroll
   for (int a = 0; a < RA; ++a) {
     acc[a][0] += o[a / W].v[a % W] * b0;
     acc[a][1] += o[a / W].v[a % W] * b1;
   }
 }
-template <typename T, int RA, int OS, int VS>
-__device__ __forceinline__ void mac(T (&acc)[8][2], const T* __restrict__ O,
-                                    const T* __restrict__ V, int kk) {
-  constexpr int BK = 64 / sizeof(T);
+template <int RA, int OS, int VS>
+__device__ __forceinline__ void mac(double (&acc)[8][2], const double* __restrict__ O,
+                                    const double* __restrict__ V, int kk) {
   if (kk == BK) {
 #pragma unroll
-    for (int k = 0; k < BK; ++k) mac_k<T, RA, OS, VS>(acc, O, V, k);
+    for (int k = 0; k < BK; ++k) mac_k<RA, OS, VS>(acc, O, V, k);
   } else {
-    for (int k = 0; k < kk; ++k) mac_k<T, RA, OS, VS>(acc, O, V, k);
+    for (int k = 0; k < kk; ++k) mac_k<RA, OS, VS>(acc, O, V, k);
   }
 }
 
 // One item with RG row groups (RG x 64 / CG long indices); Os, Vs: the CTA's tiles.
-template <typename T, int PASS, int RG>
-__device__ __forceinline__ void long_item(const T* __restrict__ v, T* __restrict__ y,
-                                          const T* __restrict__ op, const LItem& it,
+template <int PASS, int RG>
+__device__ __forceinline__ void long_item(const double* __restrict__ v, double* __restrict__ y,
+                                          const double* __restrict__ op, const LItem& it,
                                           const LSeg& sg, const LK* __restrict__ ks,
-                                          T* __restrict__ Os, T* __restrict__ Vs) {
-  constexpr int BK = 64 / sizeof(T);
+                                          double* __restrict__ Os, double* __restrict__ Vs) {
   constexpr int CG = 8 / RG, TN = 64 * CG;
   constexpr int OS = LP_ROWS;            // operator tile: [k][8 slots per row group]
   constexpr int NV = BK * TN / LT;       // V elements per thread and chunk
@@ -82,35 +79,35 @@ __device__ __forceinline__ void long_item(const T* __restrict__ v, T* __restrict
   const int mine = cg * 64 < nx ? max(0, min(ra, it.cnt - rg * ra)) : 0;
   const long long ld = sg.ld;
 
-  T acc[8][2];
+  double acc[8][2];
 #pragma unroll
-  for (int a = 0; a < 8; ++a) acc[a][0] = acc[a][1] = T(0);
+  for (int a = 0; a < 8; ++a) acc[a][0] = acc[a][1] = 0.0;
 
   // the next K chunk travels through registers while the current one is multiplied
-  T rv[NV], ro[NO];
+  double rv[NV], ro[NO];
   const int okx = tid % BK, oi = tid / BK;             // operator element of this thread
   const int vx = PASS == 0 ? tid % TN : tid / BK;      // V element: long index, k
   const int vk = PASS == 0 ? tid / TN : tid % BK;
   auto fetch = [&](const LK& k, int k0) {
     const int kk = min(BK, k.kdim - k0);
-    const T* po = op + k.op + (long long)(it.s0 + oi) * k.kdim + k0 + okx;
+    const double* po = op + k.op + (long long)(it.s0 + oi) * k.kdim + k0 + okx;
 #pragma unroll
     for (int r = 0; r < NO; ++r, po += (long long)(LT / BK) * k.kdim)
-      ro[r] = (oi + r * (LT / BK) < it.cnt && okx < kk) ? *po : T(0);
+      ro[r] = (oi + r * (LT / BK) < it.cnt && okx < kk) ? *po : 0.0;
     if (PASS == 0) {  // V(x, k): rows are contiguous
       constexpr int DX = TN > LT ? LT : 0, DK = TN > LT ? 0 : LT / TN;  // step of r
-      const T* p = v + sg.base + it.x0 + vx + ld * (k.v_off + k0 + vk);
+      const double* p = v + sg.base + it.x0 + vx + ld * (k.v_off + k0 + vk);
 #pragma unroll
       for (int r = 0; r < NV; ++r) {
         const int x = vx + (DX ? (r & 1) * LT : 0), kx = vk + (DX ? r / 2 : r * DK);
-        rv[r] = (x < nx && kx < kk) ? *p : T(0);
+        rv[r] = (x < nx && kx < kk) ? *p : 0.0;
         p += DX ? ((r & 1) ? ld - LT : LT) : ld * DK;
       }
     } else {  // V(k, x): the k of one column are contiguous
-      const T* p = v + sg.base + k.v_off + k0 + vk + ld * (it.x0 + vx);
+      const double* p = v + sg.base + k.v_off + k0 + vk + ld * (it.x0 + vx);
 #pragma unroll
       for (int r = 0; r < NV; ++r, p += ld * (LT / BK))
-        rv[r] = (vx + r * (LT / BK) < nx && vk < kk) ? *p : T(0);
+        rv[r] = (vx + r * (LT / BK) < nx && vk < kk) ? *p : 0.0;
     }
   };
   auto put = [&]() {
@@ -145,17 +142,17 @@ __device__ __forceinline__ void long_item(const T* __restrict__ v, T* __restrict
       if (++e < sg.ke) k = ks[e];
     }
     if (e < sg.ke) fetch(k, k0);
-    const T* O = Os + rg * 8;
-    const T* V = Vs + cg * 64 + lane;
+    const double* O = Os + rg * 8;
+    const double* V = Vs + cg * 64 + lane;
     switch (mine) {  // uniform in the warp
-      case 8: mac<T, 8, OS, VS>(acc, O, V, kk); break;
-      case 7: mac<T, 7, OS, VS>(acc, O, V, kk); break;
-      case 6: mac<T, 6, OS, VS>(acc, O, V, kk); break;
-      case 5: mac<T, 5, OS, VS>(acc, O, V, kk); break;
-      case 4: mac<T, 4, OS, VS>(acc, O, V, kk); break;
-      case 3: mac<T, 3, OS, VS>(acc, O, V, kk); break;
-      case 2: mac<T, 2, OS, VS>(acc, O, V, kk); break;
-      case 1: mac<T, 1, OS, VS>(acc, O, V, kk); break;
+      case 8: mac<8, OS, VS>(acc, O, V, kk); break;
+      case 7: mac<7, OS, VS>(acc, O, V, kk); break;
+      case 6: mac<6, OS, VS>(acc, O, V, kk); break;
+      case 5: mac<5, OS, VS>(acc, O, V, kk); break;
+      case 4: mac<4, OS, VS>(acc, O, V, kk); break;
+      case 3: mac<3, OS, VS>(acc, O, V, kk); break;
+      case 2: mac<2, OS, VS>(acc, O, V, kk); break;
+      case 1: mac<1, OS, VS>(acc, O, V, kk); break;
       default: break;
     }
   }
@@ -175,25 +172,24 @@ __device__ __forceinline__ void long_item(const T* __restrict__ v, T* __restrict
       }
     // the segment's padding rows, by the first row group of its last item
     if (PASS == 1 && rg == 0 && it.s0 + it.cnt == sg.dim)
-      for (int j = sg.dim; j < sg.dim_pad; ++j) y[sg.base + sg.off + j + ld * gx] = T(0);
+      for (int j = sg.dim; j < sg.dim_pad; ++j) y[sg.base + sg.off + j + ld * gx] = 0.0;
   }
 }
 
-template <typename T, int PASS>
+template <int PASS>
 __global__ void __launch_bounds__(LT, 2)
-hv_long_kernel(const T* __restrict__ v, T* __restrict__ y, const T* __restrict__ op,
+hv_long_kernel(const double* __restrict__ v, double* __restrict__ y, const double* __restrict__ op,
                const LItem* __restrict__ items, const LSeg* __restrict__ segs,
                const LK* __restrict__ ks) {
-  constexpr int BK = 64 / sizeof(T);
-  __shared__ __align__(16) T Os[BK * LP_ROWS];
-  __shared__ __align__(16) T Vs[BK * (TN_MAX + 2)];
+  __shared__ __align__(16) double Os[BK * LP_ROWS];
+  __shared__ __align__(16) double Vs[BK * (TN_MAX + 2)];
   const LItem it = items[blockIdx.x];
   const LSeg sg = segs[it.seg];
   switch (row_groups(it.cnt)) {
-    case 1: long_item<T, PASS, 1>(v, y, op, it, sg, ks, Os, Vs); break;
-    case 2: long_item<T, PASS, 2>(v, y, op, it, sg, ks, Os, Vs); break;
-    case 4: long_item<T, PASS, 4>(v, y, op, it, sg, ks, Os, Vs); break;
-    default: long_item<T, PASS, 8>(v, y, op, it, sg, ks, Os, Vs); break;
+    case 1: long_item<PASS, 1>(v, y, op, it, sg, ks, Os, Vs); break;
+    case 2: long_item<PASS, 2>(v, y, op, it, sg, ks, Os, Vs); break;
+    case 4: long_item<PASS, 4>(v, y, op, it, sg, ks, Os, Vs); break;
+    default: long_item<PASS, 8>(v, y, op, it, sg, ks, Os, Vs); break;
   }
 }
 
@@ -543,11 +539,11 @@ int lp_read_error(const LongPlan* L, int* code) {
 int lp_launch_f64(const LongPlan* L, const double* v, double* y, cudaStream_t s) {
   const int n0 = (int)L->items[0].size(), n1 = (int)L->items[1].size();
   if (n0)
-    hv_long_kernel<double, 0><<<n0, LT, 0, s>>>(v, y, L->op64[0], L->d_items[0], L->d_segs[0],
-                                                L->d_ks[0]);
+    hv_long_kernel<0><<<n0, LT, 0, s>>>(v, y, L->op64[0], L->d_items[0], L->d_segs[0],
+                                        L->d_ks[0]);
   if (n1)
-    hv_long_kernel<double, 1><<<n1, LT, 0, s>>>(v, y, L->op64[1], L->d_items[1], L->d_segs[1],
-                                                L->d_ks[1]);
+    hv_long_kernel<1><<<n1, LT, 0, s>>>(v, y, L->op64[1], L->d_items[1], L->d_segs[1],
+                                        L->d_ks[1]);
   D2_CUDA(cudaGetLastError());
   return DMRG2D_OK;
 }

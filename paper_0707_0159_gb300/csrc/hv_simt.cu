@@ -1,8 +1,10 @@
 // Superblock H·v on CUDA cores (FP64 DFMA or FP32 FMA), and the apply_H entry point.
 //
-// One CTA computes a BM x BN piece of one output tile (i2, i3) of
 //     Y = H_l V + V H_r^T + sum_k A_k V B_k^T        (paper, text after Eq. (dec))
-// in three phases that share one register accumulator:
+//
+// Dense superblocks take pieces (this file) or the two-pass kernels (hv_long.cu: V H_r^T, then
+// H_l V added, then the scalar moves added), by simt_choice.h.  In pieces, one CTA computes a
+// BM x BN piece of one output tile (i2, i3) in three phases that share one register accumulator:
 //   1. H_l V:    for every block (i2, i2') of H_l:  acc += HL[i2,i2'] * V_tile(i2', i3)
 //   2. V H_r^T:  for every block (i3, i3') of H_r:  acc += V_tile(i2, i3') * HR[i3,i3']^T
 //   3. scalar moves (H_c and off-diagonal column terms): acc += c * V_tile(i2', i3')
@@ -283,7 +285,7 @@ int launch(const dmrg2d_ops* ops, const T* v, T* y, const T* HL, const T* HR, co
     hv_simt_kernel<T, 32, 32><<<grid, TX * TY, 0, s>>>(v, y, HL, HR, C, p);
   else if (tb == 16)
     hv_simt_small_kernel<T, 16><<<grid, 256, 0, s>>>(v, y, HL, HR, C, p);
-  else
+  else if constexpr (sizeof(T) == 8)  // FP64 only (simt_choice.h)
     hv_simt_small_kernel<T, 8><<<grid, 64, 0, s>>>(v, y, HL, HR, C, p);
   D2_CUDA(cudaGetLastError());
   if (ev.second) D2_CUDA(cudaEventRecord(ev.second, s));

@@ -141,7 +141,7 @@ __global__ void k_lz_axpy2(double* __restrict__ w, const double* __restrict__ qj
 // are grid barriers of one cooperative launch (each CTA then adds the partial sums of all
 // CTAs in the same order).  As separate kernels the step was twelve launches of a few
 // microseconds each: 124 us next to an H·v of 66 us on the 2-leg m = 64 superblock (n = 65536,
-// 40 steps); in one kernel 48 us.
+// 40 steps); in one kernel 39 us.
 // The FP64 pipe (2 operations per clock and SM) makes every redundant addition count: sums
 // over a CTA or the grid are finished by one warp.
 constexpr int LZ_T = 512, LZ_CHUNK = 5120;  // threads; vector elements per CTA at most

@@ -78,15 +78,14 @@ __device__ __forceinline__ uint64_t sdesc(uint32_t addr, uint32_t lbo, uint32_t 
   return d;
 }
 // The role warps of a kernel run their loops as whole warps and issue TMA and MMA in
-// `if (elected)` blocks.  These instructions take their operands from uniform registers; where
-// the compiler can see that warp index, loop state and addresses are the warp's own, they are
-// computed there, otherwise each operand is moved over, one instruction after another.  Cycles
-// an instruction, segment kernel, TF32: MMA 84 -> 42, TMA 110 .. 125 -> 45 (a guard predicate on
-// each MMA, without the block: 84).  H·v: dense TF32 3-leg Heisenberg m = 256 43.1 -> 37.2 us,
-// BF16 m = 512 117.9 -> 101.9 us, 2-leg Hubbard m = 384 TF32 525 -> 484 us; FP64X 3-leg Hubbard
-// m = 128 10.40 -> 9.65 ms.
+// `if (elected)` blocks, with warp index, loop state and addresses written as values of the warp
+// (warp_index, bcast_uniform) instead of a thread's.  What that gives is a measured effect.
+// Cycles an instruction by clock counters, segment kernel, TF32: MMA 84 -> 42, TMA 110 .. 125 ->
+// 45 (a guard predicate on each MMA, without the block: 84).  H·v: dense TF32 3-leg Heisenberg
+// m = 256 43.1 -> 37.2 us, BF16 m = 512 117.9 -> 101.9 us, 2-leg Hubbard m = 384 TF32 525 -> 484
+// us; FP64X (seven digits) 3-leg Hubbard m = 128 10.40 -> 9.65 ms.
 
-// the warp's index, through a shuffle: uniform for the compiler, so the roles' branches are
+// the warp's index, through a shuffle
 __device__ __forceinline__ int warp_index() {
   return __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0);
 }
@@ -97,8 +96,7 @@ __device__ __forceinline__ uint32_t elect_one() {
                : "=r"(el));
   return el;
 }
-// lane `src`'s value, through a warp reduction: the result is uniform for the compiler too
-// (a shuffle's is not), so that what is computed from it stays in uniform registers
+// lane `src`'s value in all lanes, through a warp reduction
 __device__ __forceinline__ int bcast_uniform(int v, int src, int lane) {
   return (int)__reduce_or_sync(0xffffffffu, lane == src ? (unsigned)v : 0u);
 }
