@@ -296,8 +296,8 @@ int dmrg2d_lanczos_ground_noalloc(const dmrg2d_ops* ops, const dmrg2d_solver_opt
  * per block of rows (same shared-memory image, same results); 25 and 26 are configuration
  * 23 with the output tiles visited in 4 x 4 / 16 x 16 patches instead of 8 x 8.
  * dmrg2d_autotune times a complete H·v (scalar moves included) with every
- * configuration that applies (one warm-up and three timed launches each, on scratch
- * buffers it allocates and frees), keeps the fastest for later apply_H and solver
+ * configuration that applies (one warm-up and three timed launches each: their mean, or
+ * the best of them below 0.2 ms; on scratch buffers it allocates and frees), keeps the fastest for later apply_H and solver
  * calls at `precision` (TF32 or BF16), and returns its index in *best; ms[i]
  * (optional, n_ms entries) receives candidate i's time, -1 when it does not apply.
  * The call synchronises the stream.  dmrg2d_set_tile_config makes an explicit choice
