@@ -44,12 +44,24 @@ METRIC = "superblock H·v TFLOP/s & time to ground energy at 1e-8 rel. vs plain 
 # `traffic` is reported as null when the device part of csrc/hv_tc.cu (everything before
 # its host-side section) together with csrc/tc_ptx.cuh no longer has this SHA-256.
 NCU_TRAFFIC = {
-    "kernel sha256": "d49bf130d81d1a0bdd43a4515dc1382c9e7a80cca9432f14a5533abd182f5af8",
+    "kernel sha256": "cc62e60d7a05d7779ad09116e4b8d7afe89a6d279be4342ec80e9aa6044bc5d4",
     "bytes": {
+        "CTA-pair kernel 256x256 (8x8-tile blocked raster), operator pool|tf32":
+            15.54e9 + 1.07e9,
+        "CTA-pair kernel 256x256 (8x8-tile blocked raster)|tf32": 16.36e9 + 1.07e9,
         "CTA-pair kernel 256x256 (8x8-tile blocked raster), phase-2 V in one 3-D copy|tf32":
-            15.21e9 + 1.07e9,
+            16.58e9 + 1.07e9,
+        "CTA-pair kernel 256x256 (8x8-tile blocked raster), operator pool|bf16":
+            6.84e9 + 1.06e9,
+        "CTA-pair kernel 256x256 (4x4-tile blocked raster), phase-2 V in one 3-D copy|bf16":
+            8.35e9 + 1.06e9,
+        "CTA-pair kernel 256x256 (16x16-tile blocked raster), phase-2 V in one 3-D copy|bf16":
+            7.82e9 + 1.06e9,
+        "dense kernel 128x256, deduplicated operator pool|bf16": 6.55e9 + 1.06e9,
+        "dense kernel 128x256 (8x8-tile blocked raster)|bf16": 7.79e9 + 1.06e9,
+        "dense kernel 128x256 (8x8-tile blocked raster), operator pool|bf16": 6.27e9 + 1.06e9,
         "dense kernel 128x256 (8x8-tile blocked raster), phase-2 V in one 3-D copy|bf16":
-            6.81e9 + 1.06e9,
+            7.61e9 + 1.06e9,
     },
 }
 

@@ -378,9 +378,9 @@ __device__ __forceinline__ void load4(const Tin* p, int n, Tout (&o)[4]) {
   }
 }
 
-// Y(block) += sum_moves c * V(source block).  Bound by memory: a thread takes four rows of
-// one column (sector segments start at multiples of 8 rows, so the fours of an aligned
-// vector are aligned) and walks the block's moves with their addresses precomputed.  The
+// Y(block) += sum_moves c * V(source block).  Bound by memory in FP32 and BF16, in FP64 by the
+// FP64 pipe (93 .. 95 % busy): a thread takes four rows of one column (sector segments start at
+// multiples of 8 rows, so the fours of an aligned vector are aligned) and walks the block's moves with their addresses precomputed.  The
 // earlier form (one row per thread of 256, eight columns, three dependent table reads per
 // move) left most lanes of a small sector idle: on the 4-leg Heisenberg sectors of m = 1024
 // the whole BF16 H·v went from 958 to 675 us, on the 3-leg Hubbard ones in TF32 from 5.92
