@@ -1210,6 +1210,17 @@ static int tc_run_candidate(dmrg2d_ops* ops, const void* v, float* y, int prec, 
   return st;
 }
 
+// words of +-[1, 2) as FP32 (10 bits behind the point, exact in TF32), or of two BF16 each
+static __global__ void k_fill_words(uint32_t* __restrict__ w, int64_t n, uint32_t keep,
+                                    uint32_t set) {
+  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n;
+       i += (int64_t)gridDim.x * blockDim.x) {
+    uint64_t h = (uint64_t)i * 0x9e3779b97f4a7c15ull;  // a 64-bit multiplicative hash
+    h ^= h >> 32;
+    w[i] = ((uint32_t)(h * 0xd6e8feb86659fd93ull >> 32) & keep) | set;
+  }
+}
+
 }  // namespace dmrg2d
 
 using namespace dmrg2d;
@@ -1275,7 +1286,13 @@ extern "C" int dmrg2d_autotune(dmrg2d_ops* ops, int precision, int* best, double
       cudaFree(b);
     }
   } fr{v, y};
-  D2_CUDA(cudaMemsetAsync(v, 0x3C, n * (bf ? 2 : 4), s));  // small positive values
+  // Values that differ, as a vector's do: on one repeated value some candidates run several
+  // per cent faster than in use.  3-leg Hubbard m = 256, TF32: grouped column-slab 2.76 ms on a
+  // constant and 2.90 on N(0, 1) entries, CTA pair with the pool 2.77 and 2.71.
+  D2_CUDA(cudaMemsetAsync(v, 0, n * (bf ? 2 : 4), s));
+  k_fill_words<<<1024, 256, 0, s>>>((uint32_t*)v, (int64_t)(bf ? n / 2 : n),
+                                    bf ? 0x807f807fu : 0x807fe000u, bf ? 0x3f803f80u : 0x3f800000u);
+  D2_CUDA(cudaGetLastError());
   cudaEvent_t e0, e1;
   D2_CUDA(cudaEventCreate(&e0));
   D2_CUDA(cudaEventCreate(&e1));
@@ -1307,9 +1324,8 @@ extern "C" int dmrg2d_autotune(dmrg2d_ops* ops, int precision, int* best, double
         tmin = x < tmin ? x : tmin;
         tsum += x;
       }
-      // The mean of long runs: the grouped column-slab layout takes 2.7 or 2.9 ms from launch to
-      // launch on the 3-leg Hubbard m = 256 superblock, and by its best of three runs could win
-      // over a steady 2.71 ms.  The best of short runs, where launches jitter.
+      // The mean of long runs (the column-slab layout above varies by 7 % from launch to launch),
+      // the best of short ones, where launches jitter.
       t = tmin > 0.2f ? tsum / 3 : tmin;
       if (st == DMRG2D_OK && t < tbest) {
         tbest = t;
